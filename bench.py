@@ -449,10 +449,9 @@ def run_ours(args, w):
     kernel_name = {L.LACACHE_STAGE1_TENSOR: "tensor", L.LACACHE_STAGE1_TENSOR_PAIR: "tensor-pair",
                    L.LACACHE_STAGE1_STREAM: "stream", L.LACACHE_STAGE1_LSH: "lsh",
                    L.LACACHE_STAGE1_LSH_TENSOR: "lsh-tensor"}[cache.last_launch()[1]]
-    # what a step streams: the SimHash index (bits / 8 bytes an entry for the popcount scan, bits bytes for the
-    # tensor-core scan's expanded copy) or the keys
+    # what a step streams: the SimHash index (bits / 8 bytes an entry) or the keys
     if lsh:
-        flush = L2Flush(w.n * lsh["bits"] // (1 if kernel_name == "lsh-tensor" else 8), "SimHash index bytes")
+        flush = L2Flush(w.n * lsh["bits"] // 8, "SimHash index bytes")
     else:
         flush = L2Flush(w.n * w.d * 2, "keys")
     if world > 1:
@@ -565,9 +564,10 @@ def run_ours(args, w):
     # tensor pipe; a kernel timed back to back for over a second is compared with the sustained bf16 peak
     ridge = peaks["bf16_tflops"] * 1e12 / (peaks["hbm_gbs"] * 1e9)
     if lsh and kernel_name == "lsh-tensor":
-        # The tensor-core SimHash scan streams the expanded index, N x bits bytes per lookup (one byte per signature
-        # bit), and is bound by HBM; the admitted key rows it gathers are not counted.
-        index_bytes = w.n * lsh["bits"]
+        # The tensor-core SimHash scan streams the packed index, N x bits / 8 bytes per lookup; the admitted key rows
+        # it gathers are not counted. HBM is the roofline, and the scan is well below it: its warps' instruction
+        # issue binds it.
+        index_bytes = w.n * lsh["bits"] // 8
         roof = {"bound": "hbm", "achieved": index_bytes / t1_avg_s / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "peak_source": f"{peak_src} (copy bandwidth)", "algorithmic_index_bytes_per_launch": index_bytes}
     elif lsh:

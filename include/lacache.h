@@ -197,9 +197,7 @@ lacache_status lacache_append_misses(lacache_t* h, int32_t B, const void* q_emb_
  * differs from the query's in at most `radius` bits; stage 2 is unchanged. Existing entries are signed now and
  * later inserts and appends are signed as they arrive. Batches of fewer than T queries (T = 48 at 256 bits, 40 at
  * 128 and 512) compare the packed signatures by population counts; larger ones run the Hamming test on the tensor
- * cores, over a copy of the signatures expanded to one byte per bit. Allocates (capacity + max_batch) * bits / 8
- * bytes for the signatures and, when max_batch >= T, capacity * bits bytes (whole 128-entry blocks) for the
- * expanded copy.
+ * cores. Allocates (capacity + max_batch) * bits / 8 bytes for the signatures.
  * Asynchronous on cuda_stream; calling it again replaces the index. A lookup on a handle whose cfg->stage1 is
  * LACACHE_STAGE1_LSH returns LACACHE_ERR_INVALID_ARG, and runs nothing, until this call has been made. */
 lacache_status lacache_enable_lsh(lacache_t* h, int32_t bits, int32_t radius, const void* hyperplanes_dev,

@@ -152,10 +152,8 @@ struct LshArgs {
   const uint32_t* qsig;    // [B x words] query signatures
   int words;
   int radius;
-  const uint8_t* index;    // the same signatures as e4m3 +-1 bytes in swizzled 128-entry blocks (lsh_tc.cu)
 };
-// Popcount scan (small batches) and the tensor-core scan over the expanded index (batches of at least
-// lsh_tensor_min_batch(bits) queries).
+// Popcount scan (small batches) and the tensor-core scan (batches of at least lsh_tensor_min_batch(bits) queries).
 // *ring: the launch runs the scan's shared-memory ring form (the only form with bounded waits, so the only one a
 // stall injection, a.inject_stall, acts on).
 cudaError_t launch_stage1_lsh(const Stage1Args& a, const LshArgs& l, int num_sms, int max_splits, cudaStream_t st,
@@ -167,11 +165,6 @@ cudaError_t launch_stage1_lsh_tc(const Stage1Args& a, const LshArgs& l, int num_
 // B = 48 81.6 / 81.6, B = 64 97.5 / 82.4; 512 bits, B = 32 77.5 / 97.6, B = 40 104.2 / 98.9. Past 32 queries the
 // popcount scan makes a second pass over the index.
 inline int lsh_tensor_min_batch(int bits) { return bits == 256 ? 48 : 40; }
-// Bytes of the expanded index for `capacity` entries (whole 128-entry blocks of `bits` bytes each), and its update
-// from the packed signatures of entries [first, first + n).
-size_t lsh_index_bytes(int64_t capacity, int bits);
-cudaError_t launch_expand_signatures(const uint32_t* sig, int64_t first, int64_t n, int bits, uint8_t* index,
-                                     int num_sms, cudaStream_t st);
 
 // LACACHE_STAGE1_AUTO's choice for a lookup of B queries against n keys of d elements, from measurements of both
 // kernels. Once the keys stream from HBM, the tensor-core scan holds the copy bandwidth at every batch size (1.05-1.09

@@ -169,6 +169,29 @@ def test_full_radius_equals_the_exact_scan_and_appends_are_signed(batch, bits):
     assert not np.any((_unpack(sig.cpu().numpy().view(np.uint32), bits) != want) & ~amb)
 
 
+@pytest.mark.parametrize("n", [1, 127, 129, 255, 2_200, 38_913])
+@pytest.mark.parametrize("bits,batch", [(128, 129), (256, 48), (256, 300), (512, 97)])
+def test_tensor_scan_block_and_pass_edges_equal_the_exact_scan(bits, batch, n):
+    # the tensor-core scan at the edges of its 128-entry blocks and 8 KB stages (a ragged last block, one block per
+    # split, 38,913 entries = 2 blocks on all splits and 3 on some), of its 128-query passes and of its 32-query
+    # column chunks; radius = bits admits every pair, so the lookup is the exact scan's and the queue runs over
+    w = wl.WORKLOADS["mid-1m"].scaled(n=n, d=64, batch=batch, clusters=8)
+    R = wl.hyperplanes(bits, w.d, device="cuda")
+    with new_cache(w, L.LACACHE_STAGE1_TENSOR) as exact_cache, new_cache(w, L.LACACHE_STAGE1_LSH) as cache:
+        fill(exact_cache, w)
+        fill(cache, w)
+        L.lacache_enable_lsh(cache.h, bits, bits, R)
+        q = wl.batch(w, 0, device="cuda")
+        a = exact_cache.lookup(q["emb"], q["prefix"], q["ids"])
+        b = cache.lookup(q["emb"], q["prefix"], q["ids"])
+        cache.sync()
+        assert cache.last_launch()[1] == L.LACACHE_STAGE1_LSH_TENSOR
+        # fp32 sums of 64 products of bf16 unit rows in two orders: |difference| <= 64 * 2^-24 * sum |x y| < 4e-6
+        assert torch.equal(a["n_cand"], b["n_cand"])
+        assert torch.allclose(a["key_score"], b["key_score"], rtol=0, atol=4e-6)
+        assert torch.allclose(a["cand_score"], b["cand_score"], rtol=0, atol=4e-6, equal_nan=True)
+
+
 @pytest.mark.parametrize("batch", [8, 64], ids=["popcount", "tensor"])
 def test_host_buffer_lookups_through_the_index_match_device_lookups(batch):
     # inputs from mapped pinned host memory: the gather kernel writes them, the query-signature kernel waits for
