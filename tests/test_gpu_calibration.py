@@ -58,6 +58,19 @@ def test_benign_pairs_match_the_oracle(n, pct, cap):
     assert res[0] == oracle.nearest_rank(sims.astype(np.float64), pct)
 
 
+@pytest.mark.parametrize("n", [2, 1_023, 1_025, 16_384, 16_385, 131_072, 131_073])
+def test_percentile_at_the_select_kernels_limits(n):
+    # one CTA holds up to 16,384 similarities, a cluster of eight up to 131,072, more take a count and a pick per pass;
+    # dimension 8 rows of few distinct values of either sign give many ties
+    g = torch.Generator(device="cuda").manual_seed(n)
+    x = (torch.randint(-3, 4, (n, 8), generator=g, device="cuda") / 4).bfloat16()
+    y = (torch.randint(-3, 4, (n, 8), generator=g, device="cuda") / 4).bfloat16()
+    for pct in (0, 0.01, 10, 50, 99.9, 100):
+        sims, res = _gpu(x, y, pct, 0.5)
+        assert res[0] == oracle.nearest_rank(sims.astype(np.float64), pct), pct
+        assert res[1] == min(np.float32(0.5), res[0])
+
+
 def test_ties_and_invalid_arguments():
     x = torch.tensor(np.eye(8)[[0] * 64], dtype=torch.bfloat16, device="cuda")
     sims, res = _gpu(x, x, 37.5, 0.9)
