@@ -79,7 +79,8 @@ struct TcParams {
   int units;
   int64_t n_tiles;
   int k_steps;
-  int a_rows;     // rows of the query box: B rounded up to 8 when B <= 128, else 128
+  int last_mmas;  // MMAs (K = 16) of a row's last k-step: those that cover its elements
+  int last_rows;  // rows of the last query tile's box: its queries rounded up to 8
   int inject_stall;  // test support: CTA 0 withholds its second load, so its MMA issuer's bounded wait runs out
   int* tile_ctr;      // dynamic schedule: [next tile, CTAs done], zero at launch and left zero (nullptr: static)
   int wait_first;     // wait for the preceding grids before reading anything (they write the queries)
@@ -200,8 +201,8 @@ struct TopC {
 // PAIR = true: launched as two-CTA clusters, static schedule over (query-tile pair, split) units.
 template <int CPAD, bool SIGN, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
-    stage1_tensor_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
-                         const TcParams p) {
+    stage1_tensor_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_l,
+                         const __grid_constant__ CUtensorMap tmap_k, const TcParams p) {
   using G = Geo<PAIR>;
   constexpr int S = G::kStages;
   extern __shared__ unsigned char smem_raw[];
@@ -224,7 +225,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   auto tid_full_bar = [&](int r) { return bar0 + 8u * (2 * S + 5 + r); };
   auto tid_empty_bar = [&](int r) { return bar0 + 8u * (2 * S + 5 + RING + r); };
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: uniform
   const uint32_t rank = PAIR ? cluster_rank() : 0u;   // 0: leader (issues the MMAs)
 
   if (threadIdx.x == 0) {
@@ -247,6 +248,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmap_q);
+    tma_prefetch_desc(&tmap_l);
     tma_prefetch_desc(&tmap_k);
   }
   // A pair: both CTAs' barriers are initialised, and both CTAs are running, before either touches the other's
@@ -288,6 +290,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int ustep = PAIR ? (int)cluster_count_x() : (int)gridDim.x;
   const int per_split = PAIR ? p.pairs : p.q_tiles;
   auto unit_qt = [&](int u) { return PAIR ? 2 * (u % p.pairs) + (int)rank : u % p.q_tiles; };
+  // Query tile qt's box: 128 rows (tmap_q), the last tile's as many as it has queries (tmap_l), none for an odd tile
+  // count's missing partner. The MMA then also computes rows of stale shared memory, which land in TMEM lanes that the
+  // epilogue never reads. (A box of rows out of bounds is filled slowly: with one for every last tile, 129 queries on
+  // 2.4M x 384 took 512 us, and 256 queries 356.)
+  auto tile_rows = [&](int qt) { return qt + 1 < p.q_tiles ? BM : qt < p.q_tiles ? p.last_rows : 0; };
 
   if (warp == 0) {
     if (lane == 0) {
@@ -305,30 +312,31 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           if (it == withheld) continue;   // nothing arrives on this stage: its consumer's wait runs out
           if constexpr (PAIR) {
-            // both CTAs' boxes complete the leader's full barrier, which expects the bytes of all four. A box
-            // that would lie wholly out of bounds (the odd query tile's partner, the upper half of a last key
-            // tile of at most 128 keys) is replaced by the leader's box: the epilogue never reads those rows
-            // (queries >= B) or columns (ids >= n).
+            // both CTAs' boxes complete the leader's full barrier, which expects the bytes of all four. A key box
+            // that would lie wholly out of bounds (the upper half of a last key tile of at most 128 keys) is
+            // replaced by the leader's: the epilogue never reads those columns (ids >= n).
             const uint32_t lead_full = map_to_rank(full_bar(s), 0);
-            if (rank == 0) mbar_expect_tx(full_bar(s), (uint32_t)(2 * G::kStageBytes));
-            const int qy = (qt < p.q_tiles ? qt : qt - 1) * BM;
+            if (rank == 0)
+              mbar_expect_tx(full_bar(s), (uint32_t)((tile_rows(qt) + tile_rows(qt + 1)) * BK * 2 + 2 * G::kBBytes));
             const int64_t ky = t * BN + (int64_t)rank * G::kBRows;
-            tma_load_2d_pair(a_smem + s * A_BYTES, &tmap_q, lead_full, ks * BK, qy);
+            if (qt < p.q_tiles)
+              tma_load_2d_pair(a_smem + s * A_BYTES, qt + 1 < p.q_tiles ? &tmap_q : &tmap_l, lead_full, ks * BK, qt * BM);
             tma_load_2d_pair(b_smem + s * G::kBBytes, &tmap_k, lead_full, ks * BK, (int)(ky < p.n ? ky : t * BN));
           } else {
-            mbar_expect_tx(full_bar(s), (uint32_t)(p.a_rows * BK * 2 + G::kBBytes));
-            tma_load_2d(a_smem + s * A_BYTES, &tmap_q, full_bar(s), ks * BK, qt * BM);
+            mbar_expect_tx(full_bar(s), (uint32_t)(tile_rows(qt) * BK * 2 + G::kBBytes));
+            tma_load_2d(a_smem + s * A_BYTES, qt + 1 < p.q_tiles ? &tmap_q : &tmap_l, full_bar(s), ks * BK, qt * BM);
             tma_load_2d(b_smem + s * G::kBBytes, &tmap_k, full_bar(s), ks * BK, (int)(t * BN));
           }
         }
         return true;
       };
       if (dyn) {
-        int64_t next = atomicAdd(p.tile_ctr, 1);
+        // the first tile is the CTA's own: no round trip to the counter before the first load
+        int64_t next = blockIdx.x;
         for (uint32_t r = 0; ok; ++r) {
           const int64_t t = next;
           const bool done = t >= p.n_tiles;
-          if (!done) next = atomicAdd(p.tile_ctr, 1);   // claim one ahead: hides the atomic's latency
+          if (!done) next = (int64_t)gridDim.x + atomicAdd(p.tile_ctr, 1);   // one ahead: hides the atomic's latency
           const int slot = r % RING;
           if (!mbar_wait(tid_empty_bar(slot), ((r / RING) & 1u) ^ 1u, abort_flag)) {
             fail();
@@ -369,45 +377,52 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
-      // ---------------- MMA issuer ----------------
+    if (rank == 0) {
+      // ---------------- MMA issuer (the whole warp runs the loop, one lane issues: see elect_one) ----------------
       uint32_t it = 0, tile_i = 0;
       bool ok = true;
       auto mma_tile = [&]() -> bool {
         const int b = tile_i & 1u;
-        if (!mbar_wait(tempty_bar(b), ((tile_i >> 1) & 1u) ^ 1u, abort_flag)) {
-          fail();
+        if (!__all_sync(0xffffffffu, mbar_wait(tempty_bar(b), ((tile_i >> 1) & 1u) ^ 1u, abort_flag))) {
+          if (lane == 0) fail();
           return false;
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem + (uint32_t)(b * BN);
         for (int ks = 0; ks < p.k_steps; ++ks, ++it) {
           const int s = it % S;
-          if (!mbar_wait(full_bar(s), (it / S) & 1u, abort_flag)) {
-            fail();
+          if (!__all_sync(0xffffffffu, mbar_wait(full_bar(s), (it / S) & 1u, abort_flag))) {
+            if (lane == 0) fail();
             return false;
           }
           tc_fence_after();
           const uint64_t ad = smem_desc(a_smem + s * A_BYTES);
           const uint64_t bd = smem_desc(b_smem + s * G::kBBytes);
+          // the last k-step of rows that do not end on a 64-element boundary: only the MMAs that meet data
+          const int n_mma = ks + 1 < p.k_steps ? BK / 16 : p.last_mmas;
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk)
-            mma_bf16<PAIR>(d_tmem, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), (ks | kk) != 0 ? 1u : 0u);
-          mma_commit<PAIR>(empty_bar(s), 3);
+            for (int kk = 0; kk < BK / 16; ++kk)
+              if (kk < n_mma)
+                mma_bf16<PAIR>(d_tmem, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), (ks | kk) != 0 ? 1u : 0u);
+            mma_commit<PAIR>(empty_bar(s), 3);
+            if (ks + 1 == p.k_steps) mma_commit<PAIR>(tfull_bar(b), 3);
+          }
+          __syncwarp();
         }
-        mma_commit<PAIR>(tfull_bar(b), 3);
         ++tile_i;
         return true;
       };
       if (dyn) {
         for (uint32_t r = 0; ok; ++r) {
           const int slot = r % RING;
-          if (!mbar_wait(tid_full_bar(slot), (r / RING) & 1u, abort_flag)) {
-            fail();
+          if (!__all_sync(0xffffffffu, mbar_wait(tid_full_bar(slot), (r / RING) & 1u, abort_flag))) {
+            if (lane == 0) fail();
             break;
           }
           const int t = tid_ring[slot];
-          mbar_arrive(tid_empty_bar(slot));
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tid_empty_bar(slot));
           if (t < 0) break;
           ok = mma_tile();
         }
@@ -419,7 +434,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       // drain: every MMA issued by this thread has completed before TMEM is freed
-      mma_commit<PAIR>(drain_bar, 1);
+      if (elect_one()) mma_commit<PAIR>(drain_bar, 1);
+      __syncwarp();
       if (!mbar_wait(drain_bar, 0, nullptr)) fail();
       // a pair: the peer's epilogue releases of the last accumulators (remote arrivals on this CTA's barriers)
       // have landed before the leader may exit
@@ -485,9 +501,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int e = 0; e < 32; ++e)
               if (jc + e >= p.n) v[e] = -INFINITY;
           }
-          float m = v[0];
+          float mx[16];   // a tree: a chain of 31 maxima would be the chunk's longest dependency
 #pragma unroll
-          for (int e = 1; e < 32; ++e) m = fmaxf(m, v[e]);
+          for (int e = 0; e < 16; ++e) mx[e] = fmaxf(v[e], v[e + 16]);
+#pragma unroll
+          for (int w = 8; w > 0; w >>= 1)
+#pragma unroll
+            for (int e = 0; e < w; ++e) mx[e] = fmaxf(mx[e], mx[e + w]);
+          const float m = mx[0];
           best = fmaxf(best, m);
           if (m >= top.thr) {
             // rare path: stash the chunk in shared memory and insert the entries that clear the threshold
@@ -548,7 +569,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int u = unit0; ok && u < p.units; u += ustep) {
         const int qt = unit_qt(u), sp = u / per_split;
         const int q = qt * BM + row;
-        const bool active = q < p.B;
+        const bool active = qt < p.q_tiles && q < p.B;
         const int64_t t_begin = p.n_tiles * sp / p.splits, t_end = p.n_tiles * (sp + 1) / p.splits;
         const int word = (qt * BM + quad * 32) / 32;   // signature mode: this warp's word of every signature
         top.init(p.tau_c);
@@ -579,6 +600,10 @@ int gcd_int(int a, int b) {
   return a;
 }
 
+struct Maps {
+  CUtensorMap q, last, k;   // query tile, last query tile, key tile
+};
+
 template <int CPAD, bool SIGN, bool PAIR>
 cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
@@ -598,13 +623,13 @@ cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, cudaS
 }
 
 template <int CPAD, bool SIGN, bool PAIR>
-cudaError_t launch_cpad(const CUtensorMap* tq, const CUtensorMap* tk, const TcParams& p, int grid, cudaStream_t st) {
+cudaError_t launch_cpad(const Maps& m, const TcParams& p, int grid, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(stage1_tensor_kernel<CPAD, SIGN, PAIR>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<PAIR>::kSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = launch_config<CPAD, SIGN, PAIR>(attr, grid, st);
-  e = cudaLaunchKernelEx(&cfg, stage1_tensor_kernel<CPAD, SIGN, PAIR>, *tq, *tk, p);
+  e = cudaLaunchKernelEx(&cfg, stage1_tensor_kernel<CPAD, SIGN, PAIR>, m.q, m.last, m.k, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -633,9 +658,23 @@ bool encode_rows(EncodeTiledFn encode, CUtensorMap* m, const void* base, int64_t
   const cuuint64_t strides[1] = {(cuuint64_t)d * 2};
   const cuuint32_t box[2] = {(cuuint32_t)BK, box_rows};
   const cuuint32_t estr[2] = {1, 1};
+  // L2 fetches in 256-byte pieces where rows start on them (1M x 768, 32 queries: 226 us, against 232 in 128-byte
+  // pieces), else in 128-byte pieces: a box row that straddles two 256-byte pieces would fetch both (300,007 x 392, 256
+  // queries: 76 against 66 us; 200,000 x 1000: 102 against 86)
+  const CUtensorMapL2promotion l2 = d % 128 == 0 ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
   return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, l2,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The tensor maps of `rows` queries (p.q_tiles tiles of BM) against n keys in boxes of key_rows.
+bool encode_maps(EncodeTiledFn encode, Maps* m, const TcParams& p, const void* q, int rows, const void* keys,
+                 int64_t n, uint32_t key_rows) {
+  if (!encode_rows(encode, &m->last, q, p.d, rows, (uint32_t)p.last_rows) ||
+      !encode_rows(encode, &m->k, keys, p.d, n, key_rows))
+    return false;
+  m->q = m->last;   // one tile: never used
+  return p.q_tiles == 1 || encode_rows(encode, &m->q, q, p.d, rows, (uint32_t)BM);
 }
 
 // Key check of a batch of at least two query tiles on CTA pairs; false if no pair can be resident (the caller
@@ -657,10 +696,8 @@ bool launch_pairs(TcParams p, const Stage1Args& a, EncodeTiledFn encode, int max
   }
   if (clusters < 1) return false;
   p.pairs = (p.q_tiles + 1) / 2;
-  p.a_rows = BM;
-  CUtensorMap tq, tk;
-  if (!encode_rows(encode, &tq, a.q, a.d, a.B, (uint32_t)BM) ||
-      !encode_rows(encode, &tk, a.keys, a.d, a.n, (uint32_t)Geo<true>::kBRows)) {
+  Maps m;
+  if (!encode_maps(encode, &m, p, a.q, a.B, a.keys, a.n, (uint32_t)Geo<true>::kBRows)) {
     *err = cudaErrorInvalidValue;
     return true;
   }
@@ -683,26 +720,31 @@ bool launch_pairs(TcParams p, const Stage1Args& a, EncodeTiledFn encode, int max
   p.units = p.pairs * s;
   *splits = s;
   const int grid = 2 * (p.units < clusters ? p.units : clusters);
-  *err = launch_cpad<CPAD, false, true>(&tq, &tk, p, grid, st);
+  *err = launch_cpad<CPAD, false, true>(m, p, grid, st);
   return true;
+}
+
+// Whether a batch of q_tiles query tiles runs on CTA pairs. An odd count leaves one pair's second CTA without queries.
+// Single CTAs then do less work, at a lower rate (each reads the whole key box), and win for 3 and 5 tiles where rows
+// start on 256-byte boundaries (elsewhere loads bind, and a single CTA has more of them) and every CTA has several key
+// tiles. Measured (us, pairs / single CTAs, for 3, 5, 7 and 9 query tiles): 1M x 768 429 / 390, 636 / 620, 831 / 845,
+// 1073 / 1101; 300,007 x 384 89 / 71, 127 / 107, 164 / 141, 203 / 184; 300,007 x 392 98 / 105, 142 / 166, 185 / 224,
+// 232 / 289; 200,000 x 1008 119 / 123, 173 / 185, 224 / 252, 276 / 319; 40,000 x 768 34 / 36, 45 / 58, 56 / 54, 79 / 67.
+bool use_pairs(int q_tiles, int d, int64_t n_tiles, int num_sms) {
+  if (q_tiles == 1) return false;
+  return !(q_tiles % 2 == 1 && q_tiles <= 5 && d % 128 == 0 && n_tiles >= 4 * (int64_t)num_sms);
 }
 
 template <int CPAD>
 cudaError_t launch_key_check(TcParams p, const Stage1Args& a, EncodeTiledFn encode, int num_sms, int max_splits,
                              cudaStream_t st, int* splits, bool* paired) {
   cudaError_t err = cudaSuccess;
-  if (p.q_tiles >= 2 && launch_pairs<CPAD>(p, a, encode, max_splits, st, splits, &err)) {
+  if (use_pairs(p.q_tiles, a.d, p.n_tiles, num_sms) && launch_pairs<CPAD>(p, a, encode, max_splits, st, splits, &err)) {
     if (paired) *paired = true;
     return err;
   }
-  // A batch of at most 128 queries is loaded as a box of B rows (rounded up to 8) rather than 128: boxes that
-  // are mostly out of bounds stream measurably slower. The MMA still computes 128 rows; rows past B hold stale
-  // shared memory and their TMEM lanes are never read.
-  p.a_rows = a.B >= BM ? BM : ((a.B + 7) / 8) * 8;
-  CUtensorMap tq, tk;
-  if (!encode_rows(encode, &tq, a.q, a.d, a.B, (uint32_t)p.a_rows) ||
-      !encode_rows(encode, &tk, a.keys, a.d, a.n, (uint32_t)BN))
-    return cudaErrorInvalidValue;
+  Maps m;
+  if (!encode_maps(encode, &m, p, a.q, a.B, a.keys, a.n, (uint32_t)BN)) return cudaErrorInvalidValue;
   // splits such that q_tiles * splits is a multiple of the SM count (whole waves of units); one query tile with
   // a tile counter: a dynamic schedule with one split per CTA
   int s = num_sms / gcd_int(num_sms, p.q_tiles);
@@ -714,7 +756,7 @@ cudaError_t launch_key_check(TcParams p, const Stage1Args& a, EncodeTiledFn enco
   if (p.q_tiles == 1 && a.tile_ctr) p.tile_ctr = a.tile_ctr;
   *splits = s;
   const int grid = p.units < num_sms ? p.units : num_sms;
-  return launch_cpad<CPAD, false, false>(&tq, &tk, p, grid, st);
+  return launch_cpad<CPAD, false, false>(m, p, grid, st);
 }
 
 }  // namespace
@@ -731,9 +773,10 @@ cudaError_t launch_signatures(const __nv_bfloat16* rows, int64_t n, int d, const
   p.tau_c = 0.f;
   p.top_c = 1;
   p.q_tiles = (bits + BM - 1) / BM;
+  p.last_rows = (bits - (p.q_tiles - 1) * BM + 7) / 8 * 8;
   p.n_tiles = (n + BN - 1) / BN;
   p.k_steps = (d + BK - 1) / BK;
-  p.a_rows = bits >= BM ? BM : ((bits + 7) / 8) * 8;
+  p.last_mmas = (d - (p.k_steps - 1) * BK + 15) / 16;
   int s = num_sms / gcd_int(num_sms, p.q_tiles);
   if ((int64_t)s > p.n_tiles) s = (int)p.n_tiles;
   if (s < 1) s = 1;
@@ -742,12 +785,10 @@ cudaError_t launch_signatures(const __nv_bfloat16* rows, int64_t n, int d, const
   p.sig = sig;
   p.sig_words = bits / 32;
   p.dev_status = dev_status;
-  CUtensorMap tq, tk;
-  if (!encode_rows(encode, &tq, hyperplanes, d, bits, (uint32_t)p.a_rows) ||
-      !encode_rows(encode, &tk, rows, d, n, (uint32_t)BN))
-    return cudaErrorInvalidValue;
+  Maps m;
+  if (!encode_maps(encode, &m, p, hyperplanes, bits, rows, n, (uint32_t)BN)) return cudaErrorInvalidValue;
   const int grid = p.units < num_sms ? p.units : num_sms;
-  return launch_cpad<4, true, false>(&tq, &tk, p, grid, st);
+  return launch_cpad<4, true, false>(m, p, grid, st);
 }
 
 cudaError_t launch_stage1_tensor(const Stage1Args& a, EncodeTiledFn encode, int num_sms, int max_splits,
@@ -760,8 +801,10 @@ cudaError_t launch_stage1_tensor(const Stage1Args& a, EncodeTiledFn encode, int 
   p.tau_c = a.tau_c;
   p.top_c = a.top_c;
   p.q_tiles = (a.B + BM - 1) / BM;
+  p.last_rows = (a.B - (p.q_tiles - 1) * BM + 7) / 8 * 8;
   p.n_tiles = (a.n + BN - 1) / BN;
   p.k_steps = (a.d + BK - 1) / BK;
+  p.last_mmas = (a.d - (p.k_steps - 1) * BK + 15) / 16;
   p.part_cand = a.part_cand;
   p.part_meta = a.part_meta;
   p.dev_status = a.dev_status;

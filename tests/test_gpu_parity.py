@@ -78,6 +78,25 @@ def test_ragged_batch_dimension_and_k(stage1):
     assert rep.exact + rep.band == w.batch and rep.band <= 2
 
 
+@pytest.mark.parametrize("n,d,batch,pairs", [(5_000, 392, 129, True), (5_000, 136, 250, True), (3_000, 1000, 257, True),
+                                             (160_000, 128, 257, False), (160_000, 128, 520, False),
+                                             (160_000, 128, 769, True), (160_000, 136, 257, True)])
+def test_query_tile_edges_and_odd_tile_counts(n, d, batch, pairs):
+    # a last query tile of 1, 2, 8 and 122 queries (its box has as many rows, in eights), rows whose last k-step holds
+    # one MMA's elements (d = 8 mod 64), and odd counts of query tiles, on single CTAs for 3 and 5 of them where rows
+    # start on 256-byte boundaries and the store has at least four key tiles per SM (155,648 entries on 152 SMs)
+    w = wl.WORKLOADS["mid-1m"].scaled(n=n, d=d, batch=batch, clusters=64)
+    st = oracle_store(w)
+    with new_cache(w, L.LACACHE_STAGE1_TENSOR) as cache:
+        fill(cache, w)
+        q = wl.batch(w, 0, device="cuda")
+        g = gpu_lookup(cache, q)
+        assert cache.last_launch()[1] == (L.LACACHE_STAGE1_TENSOR_PAIR if pairs else L.LACACHE_STAGE1_TENSOR)
+    oq, p = oracle_queries(q), params(w)
+    rep = compare(g, oracle.lookup(st, oq, p), p, pair_scores=pair_scores_fn(st, oq))
+    assert rep.exact + rep.band == w.batch and rep.band <= w.batch // 10
+
+
 @pytest.mark.parametrize("stage1", PATHS)
 @pytest.mark.parametrize("d,k,batch", [(8, 1, 1), (8192, 256, 40)], ids=["smallest", "largest"])
 def test_dimension_and_window_extremes(stage1, d, k, batch):
