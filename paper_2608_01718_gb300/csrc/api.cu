@@ -35,7 +35,8 @@ struct lacache {
   unsigned char* stage_out;  // device staging for lookup_host results
   unsigned char* pinned;     // one mapped pinned allocation: append_count_host, then stage_host
   unsigned char* stage_host; // pinned host staging of lookup_host results (mapped: the kernels write it directly)
-  unsigned char* stage_host_dev; // device address of stage_host, or nullptr if the device cannot map it
+  unsigned char* pinned_dev;     // device address of pinned, or nullptr if the device cannot map it
+  unsigned char* stage_host_dev; // ... and of stage_host
   int last_splits;
   int last_kernel;
   lc::EncodeTiledFn encode;
@@ -135,6 +136,54 @@ __global__ void append_rows_kernel(const uint4* __restrict__ q_emb, const uint4*
   for (int i = threadIdx.x; i < kv; i += blockDim.x) key[row * kv + i] = q_emb[(int64_t)q * kv + i];
   for (int i = threadIdx.x; i < pv; i += blockDim.x) pre[row * pv + i] = q_pre[(int64_t)q * pv + i];
   for (int i = threadIdx.x; i < k; i += blockDim.x) ids[row * k + i] = q_ids[(int64_t)q * k + i];
+}
+
+// The two kernels above in one, for batches of up to kAppendFusedMax queries: each block takes kAppendQ queries, counts the
+// non-HIT queries before them and in the whole batch itself (a byte a query, from L2), and copies its rows, one warp
+// a row; block 0 writes the count straight into mapped pinned host memory. Bound by latency: one launch and no copy back,
+// for a rank kernel, a row kernel and a device-to-host copy. A call (with its synchronization, d = 768; us, before /
+// after): 1 query 25 / 18, 256 32 / 19, 8,192 35 / 26, 16,384 45 / 36. Past the limit the counting, quadratic in the
+// batch, would cost more than it saves.
+constexpr int kAppendQ = 8;
+constexpr int kAppendFusedMax = 16384;
+__global__ void __launch_bounds__(kAppendQ * 32)
+    append_fused_kernel(const uint4* __restrict__ q_emb, const uint4* __restrict__ q_pre,
+                        const int32_t* __restrict__ q_ids, const uint8_t* __restrict__ status, int B, int d, int pd,
+                        int k, int64_t n0, int64_t capacity, uint4* __restrict__ key, uint4* __restrict__ pre,
+                        int32_t* __restrict__ ids, int32_t* __restrict__ count_host) {
+  __shared__ int part[2][kAppendQ];
+  __shared__ uint8_t miss[kAppendQ];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int q0 = blockIdx.x * kAppendQ;
+  int before = 0, all = 0;
+  for (int q = threadIdx.x; q < B; q += kAppendQ * 32) {
+    const int m = __ldcg(status + q) != LACACHE_HIT ? 1 : 0;
+    all += m;
+    before += q < q0 ? m : 0;
+  }
+  before = __reduce_add_sync(0xffffffffu, before);
+  all = __reduce_add_sync(0xffffffffu, all);
+  if (lane == 0) {
+    part[0][warp] = before;
+    part[1][warp] = all;
+    miss[warp] = q0 + warp < B && __ldcg(status + q0 + warp) != LACACHE_HIT ? 1 : 0;
+  }
+  __syncthreads();
+  int rank = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kAppendQ; ++w) {
+    rank += part[0][w] + (w < warp ? miss[w] : 0);
+    total += part[1][w];
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *count_host = total;
+  if (n0 + total > capacity || !miss[warp]) return;
+  const int q = q0 + warp;
+  const int kv = d / 8, pv = pd / 8;   // 16-byte vectors per key row and per prefix row
+  const int64_t row = n0 + rank;
+  for (int i = lane; i < kv; i += 32) key[row * kv + i] = q_emb[(int64_t)q * kv + i];
+  for (int i = lane; i < pv; i += 32) pre[row * pv + i] = q_pre[(int64_t)q * pv + i];
+  for (int i = lane; i < k; i += 32) ids[row * k + i] = q_ids[(int64_t)q * k + i];
 }
 
 // lookup_host's inputs, read by the device straight from mapped pinned host memory (NVLink-C2C on Grace) into the
@@ -520,10 +569,11 @@ lacache_status lacache_create_ensemble(const lacache_config* cfg, const lacache_
     delete h;
     return LACACHE_ERR_OOM;
   }
-  if (cudaHostGetDevicePointer((void**)&h->stage_host_dev, h->stage_host, 0) != cudaSuccess) {
+  if (cudaHostGetDevicePointer((void**)&h->pinned_dev, h->pinned, 0) != cudaSuccess) {
     cudaGetLastError();
-    h->stage_host_dev = nullptr;   // results then come back with one device-to-host copy
+    h->pinned_dev = nullptr;   // results and counts then come back with a device-to-host copy
   }
+  h->stage_host_dev = h->pinned_dev ? h->pinned_dev + kPinnedCountBytes : nullptr;
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult q;
   if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) ==
@@ -695,13 +745,29 @@ lacache_status lacache_append_misses(lacache_t* h, int32_t B, const void* q_emb_
   if (!guard.ok()) return LACACHE_ERR_CUDA;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const lacache_config& c = h->cfg;
-  append_rank_kernel<<<1, 1024, 0, st>>>(status_dev, B, h->append_dst, h->append_count);
-  append_rows_kernel<<<B, 128, 0, st>>>((const uint4*)q_emb_dev, (const uint4*)q_prefix_dev, q_ids_dev,
-                                        h->append_dst, h->append_count, B, c.d, h->pd, c.k, h->n, c.capacity,
-                                        (uint4*)h->key, (uint4*)h->prefix, h->ids);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h->append_count_host, h->append_count, 4, cudaMemcpyDeviceToHost, st);
+  cudaError_t e;
+  if (B <= kAppendFusedMax && h->pinned_dev) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((B + kAppendQ - 1) / kAppendQ));
+    cfg.blockDim = dim3(kAppendQ * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, append_fused_kernel, (const uint4*)q_emb_dev, (const uint4*)q_prefix_dev, q_ids_dev,
+                           status_dev, (int)B, (int)c.d, h->pd, (int)c.k, h->n, c.capacity, (uint4*)h->key,
+                           (uint4*)h->prefix, h->ids, reinterpret_cast<int32_t*>(h->pinned_dev));
+  } else {
+    append_rank_kernel<<<1, 1024, 0, st>>>(status_dev, B, h->append_dst, h->append_count);
+    append_rows_kernel<<<B, 128, 0, st>>>((const uint4*)q_emb_dev, (const uint4*)q_prefix_dev, q_ids_dev,
+                                          h->append_dst, h->append_count, B, c.d, h->pd, c.k, h->n, c.capacity,
+                                          (uint4*)h->key, (uint4*)h->prefix, h->ids);
+    e = cudaGetLastError();
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(h->append_count_host, h->append_count, 4, cudaMemcpyDeviceToHost, st);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return LACACHE_ERR_CUDA;
   const int64_t m = *h->append_count_host;

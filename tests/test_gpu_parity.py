@@ -572,3 +572,31 @@ def test_lookup_captured_in_a_cuda_graph_replays_like_eager_lookups(stage1, batc
             cache.sync()
             for k in out:
                 assert torch.equal(out[k].view(torch.uint8), want[k].view(torch.uint8)), (step, k)
+
+
+@pytest.mark.parametrize("B", [1, 7, 8, 9, 255, 16_384, 16_385])
+def test_append_takes_the_non_hit_rows_in_query_order(B):
+    # blocks of eight queries that count the misses before them (up to 16,384 queries), and the rank and row kernels past
+    # that; then the same append on a store one row too small, which must leave it as it was
+    g = torch.Generator(device="cuda").manual_seed(B)
+    emb = torch.randn((B, 24), generator=g, device="cuda").bfloat16()
+    pre = torch.randn((B, 24), generator=g, device="cuda").bfloat16()
+    ids = torch.randint(0, 99, (B, 33), generator=g, device="cuda", dtype=torch.int32)
+    status = torch.randint(0, 3, (B,), generator=g, device="cuda").to(torch.uint8)
+    status[0] = L.LACACHE_REJECT
+    miss = status != L.LACACHE_HIT
+    m = int(miss.sum())
+    for capacity in (5 + m, 4 + m):
+        with L.LaCache(24, 33, capacity, 0.9, 0.8, 4, max_batch=B) as cache:
+            n0 = min(5, B)
+            cache.insert(emb[:n0], pre[:n0], ids[:n0])
+            if capacity < n0 + m:
+                with pytest.raises(L.LacacheError) as e:
+                    cache.append_misses(emb, pre, ids, status)
+                assert e.value.status == L.LACACHE_ERR_CAPACITY and cache.size == n0
+                continue
+            assert cache.append_misses(emb, pre, ids, status) == (n0, m) and cache.size == n0 + m
+            key, prefix, tok = torch.empty_like(emb[:m]), torch.empty_like(pre[:m]), torch.empty_like(ids[:m])
+            L.lacache_read_rows(cache.h, n0, m, key, prefix, tok)
+            cache.sync()
+            assert torch.equal(key, emb[miss]) and torch.equal(prefix, pre[miss]) and torch.equal(tok, ids[miss])
