@@ -24,7 +24,8 @@
 //     epoch; release the accumulator;
 //   warps 16-21 (checker warps): claim queued pairs as they arrive, compute their exact fp32 key scores over the
 //     gathered key rows (each lane's 8-element chunks in order, then a butterfly sum) while the scan goes on, and
-//     fold each score into its query's best score and, if it clears tau_c, into the query's list (lock-free).
+//     fold each score into its query's best score and, if it clears tau_c, into the query's list (lock-free). The
+//     mask warps join them once the range is scanned.
 // When the queue passes three quarters of its capacity, and at the end of the range, the mask warps close it: the
 // checkers finish what was queued below the close, then the queue is emptied and reopened in a new epoch. A pair
 // that finds the queue full stays with its thread and is queued after the reopening. All
@@ -39,10 +40,12 @@
 // entries at 128 queries and 256 bits; the packed index takes 20 us of HBM time on 4M entries, the MMAs 55 us. Four mask
 // warps share a block's columns, since accumulators for only three blocks fit beside the A buffers; they meet at a
 // barrier only every 32 blocks (every 8: 10 % slower); the roles' loops are rolled, to share the instruction cache.
-// Measured per lookup step, d = 768, top_c = 8, against the scan over an index kept expanded in HBM that this one
-// replaces (us, before / after): 4M entries, 256 bits, 48 queries 177 / 154, 64 180 / 156, 96 210 / 167, 128 202 / 186;
-// 128 bits, 64 queries 135 / 133, 128 184 / 175; 512 bits, 64 queries 326 / 219, 128 631 / 238; 1M entries, 256 bits, 64
-// queries 64 / 52, 128 73 / 60. The index takes an eighth of the memory, and signing entries no second kernel.
+// Measured per lookup step against the scan over an index kept expanded in HBM that this one replaces (us, before /
+// after): 4M x 768, 256 bits, 48 queries 177 / 169, 64 180 / 171, 128 202 / 184; 128 bits, 128 queries 184 / 175; 512
+// bits, 64 queries 326 / 219, 128 631 / 238; 1M x 1024, 256 bits, 128 queries 70 / 63, 357 181 / 167; 36,433 x 768, 357
+// queries 44 / 40. (Without the mask warps' help at the end of the range 48 queries on 4M x 768 take 150, but 128 on
+// 4M x 1024 take 233 instead of 198, and 357 on 36,433 x 768 take 49.) The index takes an eighth of the memory, and signing
+// entries no second kernel.
 #include "internal.cuh"
 #include "tcgen05.cuh"
 
@@ -196,7 +199,7 @@ __device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint32_t a_tmem, uint6
       : "memory");
 }
 
-// A checker warp's wait (by one lane) for queue position `slot` of epoch ep: true, with the pair, once it is there; false once the
+// A checker lane's wait for queue position `slot` of epoch ep: true, with the pair, once it is there; false once the
 // mask warps closed the queue at or below the slot (that position holds nothing to check in this epoch), or after
 // about a second (the timeout is recorded; the mask warps then see the abort flag and close the queue).
 __device__ __forceinline__ bool wait_slot(Tail& t, int slot, uint32_t ep, uint64_t* item, unsigned int* dev_status) {
@@ -241,6 +244,30 @@ __device__ __forceinline__ float check_pair(uint64_t item, const __nv_bfloat16* 
       if (c0 + 32 * i < v) acc = dot8(x[i], kv[i], acc);
   }
   return warp_sum(acc);
+}
+
+// The same for kNarrowItems pairs of rows of at most 256 elements, one chunk per lane: as many loads in flight as for one
+// wide pair. Lane u returns pair u's score. (One at a time, 357 queries on 36,433 x 160 took 47 us, and so 37.)
+constexpr int kNarrowItems = 3;
+__device__ __forceinline__ float check_narrow(const uint64_t (&item)[kNarrowItems],
+                                              const __nv_bfloat16* __restrict__ keys,
+                                              const __nv_bfloat16* __restrict__ q, int d, int q0, int lane) {
+  uint4 kv[kNarrowItems], x[kNarrowItems];
+#pragma unroll
+  for (int u = 0; u < kNarrowItems; ++u) {
+    kv[u] = x[u] = make_uint4(0u, 0u, 0u, 0u);
+    if (lane < d / 8) {
+      kv[u] = __ldg(reinterpret_cast<const uint4*>(keys + (int64_t)item_entry(item[u]) * d) + lane);
+      x[u] = __ldg(reinterpret_cast<const uint4*>(q + (int64_t)(q0 + item_query(item[u])) * d) + lane);
+    }
+  }
+  float score = 0.f;
+#pragma unroll
+  for (int u = 0; u < kNarrowItems; ++u) {
+    const float s = warp_sum(dot8(x[u], kv[u], 0.f));
+    if (lane == u) score = s;
+  }
+  return score;
 }
 
 // Fold one exact score into its query's best score and, if it clears tau_c, into the query's list (unordered, 0 =
@@ -495,14 +522,12 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
       const int mw = warp;                                 // mask warp
       const int quad = mw % 4, part = mw / 4;              // TMEM lane quadrant; column chunk(s) part + kMaskParts i
       const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
-      // close the queue (every mask warp has queued its pairs); reopen it once the checkers are done with it
-      auto close_and_reopen = [&](bool last) {
+      // close the queue (every mask warp has queued its pairs)
+      auto close = [&](bool last) {
         if (mw == 0 && lane == 0) {
           if (last) t.pass_end = 1;   // read after the reopening's barriers
           st_volatile(&t.closed, 1u + (uint32_t)min(t.count, kCap));
         }
-        reopen(t, mw, lane);
-        ++ep;
       };
       const int nch = npad / 32;                           // 32-query chunks of a block
       first_acc(it);
@@ -575,7 +600,9 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
             stop = true;
             break;
           }
-          close_and_reopen(false);
+          close(false);
+          reopen(t, mw, lane);   // once the checkers are done with it
+          ++ep;
           top = -1;
           for (uint32_t o = over; o; o &= o - 1) {
             const int i = __ffs(o) - 1;
@@ -584,23 +611,40 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
           }
         }
       }
-      // the pass's last close, also after a timeout: the checker warps leave only at a reopening
-      close_and_reopen(true);
+      // the pass's last close, also after a timeout: the checkers leave only at a reopening
+      close(true);
       it += nb;
-    } else if (warp < kEpiWarps) {
-      // ---------------- checker warps ----------------
-      // claim a queue position, check and fold its pair while the scan goes on; at a close, finish what was queued
-      // below it, then take part in the reopening
+    }
+
+    if (warp < kEpiWarps) {
+      // ---------------- checker warps, and the mask warps once the range is scanned ----------------
+      // claim a queue position (several for narrow rows), check and fold its pair while the scan goes on; at a close,
+      // finish what was queued below it, then take part in the reopening
+      const int claims = a.d <= 256 ? kNarrowItems : 1;
       for (;;) {
         for (;;) {
-          uint64_t item = 0;
-          bool there = false;
-          if (lane == 0) there = wait_slot(t, atomicAdd(&t.claim, 1), ep, &item, a.dev_status);
-          if (!__shfl_sync(kFull, (int)there, 0)) break;   // a position past the close (or a timeout)
-          item = __shfl_sync(kFull, item, 0);
-          const float score = check_pair(item, a.keys, a.q, a.d, q0, lane);
-          if (lane == 0) fold_one(t, lists, C, a.tau_c, item_query(item), item_entry(item), score);
-          __syncwarp();
+          int base = 0;
+          if (lane == 0) base = atomicAdd(&t.claim, claims);
+          base = __shfl_sync(kFull, base, 0);
+          uint64_t got = 0;
+          const bool mine = lane < claims && wait_slot(t, base + lane, ep, &got, a.dev_status);
+          const unsigned ready = __ballot_sync(kFull, mine);
+          if (ready) {
+            float score;   // lane u: of the pair at base + u
+            if (claims == 1) {
+              score = check_pair(__shfl_sync(kFull, got, 0), a.keys, a.q, a.d, q0, lane);
+            } else {
+              // a position without a pair repeats one that has it, and is not folded
+              uint64_t item[kNarrowItems];
+#pragma unroll
+              for (int u = 0; u < kNarrowItems; ++u)
+                item[u] = __shfl_sync(kFull, got, (ready >> u) & 1u ? u : __ffs(ready) - 1);
+              score = check_narrow(item, a.keys, a.q, a.d, q0, lane);
+            }
+            if (mine) fold_one(t, lists, C, a.tau_c, item_query(got), item_entry(got), score);
+            __syncwarp();
+          }
+          if (ready != (1u << claims) - 1u) break;   // a position past the close (or a timeout)
         }
         reopen(t, warp, lane);
         ++ep;
