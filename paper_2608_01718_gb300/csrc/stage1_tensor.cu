@@ -652,16 +652,20 @@ int max_pair_clusters(cudaStream_t st) {
   return clusters;
 }
 
+// `batch`: queries (or hyperplanes) of the launch.
 bool encode_rows(EncodeTiledFn encode, CUtensorMap* m, const void* base, int64_t d, int64_t rows,
-                 uint32_t box_rows) {
+                 uint32_t box_rows, int batch) {
   const cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)d * 2};
   const cuuint32_t box[2] = {(cuuint32_t)BK, box_rows};
   const cuuint32_t estr[2] = {1, 1};
-  // L2 fetches in 256-byte pieces where rows start on them (1M x 768, 32 queries: 226 us, against 232 in 128-byte
-  // pieces), else in 128-byte pieces: a box row that straddles two 256-byte pieces would fetch both (300,007 x 392, 256
-  // queries: 76 against 66 us; 200,000 x 1000: 102 against 86)
-  const CUtensorMapL2promotion l2 = d % 128 == 0 ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
+  // L2 fetches in 256-byte pieces, which HBM streams best, except where rows start off 32-byte boundaries (d = 8 mod 16)
+  // and the batch makes L2 the busier side: a box row then straddles pieces and would fetch both. Measured (us, 256-byte /
+  // 128-byte pieces): 3.6M x 968, 16 queries 961 / 996, 64 970 / 1015, 96 1005 / 1020, 128 1101 / 1027, 256 1673 / 1465, 512
+  // 3187 / 2562; 1M x 392, 16 queries 117 / 119, 64 140 / 123, 128 160 / 134, 512 413 / 345; 32-byte rows: 3M x 448, 128
+  // queries 369 / 381, 256 480 / 497.
+  const CUtensorMapL2promotion l2 =
+      d % 16 == 8 && batch >= 96 ? CU_TENSOR_MAP_L2_PROMOTION_L2_128B : CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
   return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, l2,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -670,11 +674,11 @@ bool encode_rows(EncodeTiledFn encode, CUtensorMap* m, const void* base, int64_t
 // The tensor maps of `rows` queries (p.q_tiles tiles of BM) against n keys in boxes of key_rows.
 bool encode_maps(EncodeTiledFn encode, Maps* m, const TcParams& p, const void* q, int rows, const void* keys,
                  int64_t n, uint32_t key_rows) {
-  if (!encode_rows(encode, &m->last, q, p.d, rows, (uint32_t)p.last_rows) ||
-      !encode_rows(encode, &m->k, keys, p.d, n, key_rows))
+  if (!encode_rows(encode, &m->last, q, p.d, rows, (uint32_t)p.last_rows, rows) ||
+      !encode_rows(encode, &m->k, keys, p.d, n, key_rows, rows))
     return false;
   m->q = m->last;   // one tile: never used
-  return p.q_tiles == 1 || encode_rows(encode, &m->q, q, p.d, rows, (uint32_t)BM);
+  return p.q_tiles == 1 || encode_rows(encode, &m->q, q, p.d, rows, (uint32_t)BM, rows);
 }
 
 // Key check of a batch of at least two query tiles on CTA pairs; false if no pair can be resident (the caller
