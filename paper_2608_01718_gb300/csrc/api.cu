@@ -384,9 +384,27 @@ void free_all(lacache* h) {
   if (h->pinned) cudaFreeHost(h->pinned);
 }
 
-// gathered: the queries were just written by gather_host_kernel, so the first kernel waits for it before reading.
+// The stage-1 kernel of a lookup of B queries (a lacache_stage1 value).
+int stage1_of(const lacache* h, int32_t B) {
+  return h->cfg.stage1 == LACACHE_STAGE1_AUTO ? lc::auto_stage1(h->n, h->cfg.d, B) : h->cfg.stage1;
+}
+
+// Whether the kernels of a host-buffer lookup read its inputs (device addresses of mapped host memory) where they are,
+// without the gather: for the streaming scan, each of whose CTAs reads the batch once, while that is at most
+// kDirectBytes over the link in all; the tensor scan reads the batch again for every key tile.
+constexpr size_t kDirectBytes = (size_t)1 << 20;
+bool reads_host_inputs(const lacache* h, int32_t B, const void* emb, const void* pre, const void* ids) {
+  return stage1_of(h, B) == LACACHE_STAGE1_STREAM && emb && pre && ids && aligned16(emb) && aligned16(pre) &&
+         (uintptr_t)ids % 4 == 0 && (size_t)h->num_sms * B * h->cfg.d * 2 <= kDirectBytes;
+}
+
+// Where a lookup's inputs come from: the caller's device memory, the staging that gather_host_kernel just wrote (so the
+// first kernel waits for it before reading), or mapped host memory.
+enum class Inputs { kDevice, kGathered, kHost };
+
 lacache_status run_lookup(lacache* h, int32_t B, const void* q_emb, const void* q_prefix, const int32_t* q_ids,
-                          const lacache_result& out, cudaStream_t st, bool gathered = false) {
+                          const lacache_result& out, cudaStream_t st, Inputs inputs = Inputs::kDevice) {
+  const bool gathered = inputs == Inputs::kGathered;
   const lacache_config& c = h->cfg;
   if (!lookup_ready(h)) return LACACHE_ERR_INVALID_ARG;
   int splits = 0;
@@ -407,7 +425,8 @@ lacache_status run_lookup(lacache* h, int32_t B, const void* q_emb, const void* 
     a.part_meta = h->part_meta;
     a.dev_status = h->dev_status;
     a.inputs_from_previous = gathered ? 1 : 0;
-    kernel = c.stage1 == LACACHE_STAGE1_AUTO ? lc::auto_stage1(h->n, c.d, B) : c.stage1;
+    a.q_host = inputs == Inputs::kHost ? 1 : 0;
+    kernel = stage1_of(h, B);
     if (h->inject_stall > 0 && kernel == LACACHE_STAGE1_TENSOR) {
       a.inject_stall = 1;
       --h->inject_stall;
@@ -469,6 +488,7 @@ lacache_status run_lookup(lacache* h, int32_t B, const void* q_emb, const void* 
   b.q_ids = q_ids;
   b.out = out;
   b.counters = h->counters;
+  b.host_inputs = inputs == Inputs::kHost ? 1 : 0;
   if (ev && cudaEventRecord(ev[1], st) != cudaSuccess) return LACACHE_ERR_CUDA;
   if (lc::launch_stage2(b, st) != cudaSuccess) return LACACHE_ERR_CUDA;
   if (ev && cudaEventRecord(ev[2], st) != cudaSuccess) return LACACHE_ERR_CUDA;
@@ -652,27 +672,36 @@ lacache_status lacache_lookup_host(lacache_t* h, int32_t B, const void* q_emb_ho
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const lacache_config& c = h->cfg;
   const HostInputs in = host_inputs(h, B, q_emb_host, q_prefix_host, q_ids_host);
-  next_stage_slot(h);
-  // Inputs: arrays in mapped pinned memory are gathered by one kernel; any other array is copied by DMA.
-  GatherArgs g{};
-  size_t gathered = 0;
-  for (int i = 0; i < 3; ++i) {
-    const void* dev_src = mapped_device_pointer(in.src[i]);
-    if (dev_src) {
-      g.seg[i] = GatherSeg{static_cast<const unsigned char*>(dev_src), in.dst[i], in.bytes[i]};
-      gathered += in.bytes[i];
-    } else if (cudaMemcpyAsync(in.dst[i], in.src[i], in.bytes[i], cudaMemcpyHostToDevice, st) != cudaSuccess) {
-      return LACACHE_ERR_CUDA;
+  // Inputs: arrays in mapped pinned memory are gathered by one kernel, or read where they are; any other array is copied
+  // by DMA.
+  const void* src[3];
+  for (int i = 0; i < 3; ++i) src[i] = mapped_device_pointer(in.src[i]);
+  Inputs inputs = Inputs::kDevice;
+  if (reads_host_inputs(h, B, src[0], src[1], src[2])) {
+    inputs = Inputs::kHost;
+  } else {
+    next_stage_slot(h);
+    GatherArgs g{};
+    size_t gathered = 0;
+    for (int i = 0; i < 3; ++i) {
+      if (src[i]) {
+        g.seg[i] = GatherSeg{static_cast<const unsigned char*>(src[i]), in.dst[i], in.bytes[i]};
+        gathered += in.bytes[i];
+        inputs = Inputs::kGathered;
+      } else if (cudaMemcpyAsync(in.dst[i], in.src[i], in.bytes[i], cudaMemcpyHostToDevice, st) != cudaSuccess) {
+        return LACACHE_ERR_CUDA;
+      }
+      src[i] = in.dst[i];
     }
+    if (gathered && launch_gather(h, g, gathered, st) != cudaSuccess) return LACACHE_ERR_CUDA;
   }
-  if (gathered && launch_gather(h, g, gathered, st) != cudaSuccess) return LACACHE_ERR_CUDA;
   size_t bytes = 0;
   // Results: written by the kernels straight into the mapped pinned staging when the device can map it.
   unsigned char* out_stage = h->stage_host_dev ? h->stage_host_dev : h->stage_out;
   lacache_result dev = staged_result(out_stage, B, c.top_c, h->ens.m, *out_host, &bytes);
   lacache_result host = staged_result(h->stage_host, B, c.top_c, h->ens.m, *out_host, &bytes);
   lacache_status s =
-      run_lookup(h, B, in.dst[0], in.dst[1], reinterpret_cast<const int32_t*>(in.dst[2]), dev, st, gathered != 0);
+      run_lookup(h, B, src[0], src[1], static_cast<const int32_t*>(src[2]), dev, st, inputs);
   if (s != LACACHE_OK) return s;
   if (!h->stage_host_dev &&
       cudaMemcpyAsync(h->stage_host, h->stage_out, bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess)
@@ -711,10 +740,11 @@ lacache_status lacache_lookup_host_async(lacache_t* h, int32_t B, const void* q_
   const HostInputs in = host_inputs(h, B, q_emb_host, q_prefix_host, q_ids_host);
   GatherArgs g{};
   size_t gathered = 0;
+  const void* src[3];
   for (int i = 0; i < 3; ++i) {
-    const void* dev_src = mapped_device_pointer(in.src[i]);
-    if (!dev_src) return LACACHE_ERR_INVALID_ARG;
-    g.seg[i] = GatherSeg{static_cast<const unsigned char*>(dev_src), in.dst[i], in.bytes[i]};
+    src[i] = mapped_device_pointer(in.src[i]);
+    if (!src[i]) return LACACHE_ERR_INVALID_ARG;
+    g.seg[i] = GatherSeg{static_cast<const unsigned char*>(src[i]), in.dst[i], in.bytes[i]};
     gathered += in.bytes[i];
   }
   const lacache_result& o = *out_host;
@@ -729,9 +759,12 @@ lacache_status lacache_lookup_host_async(lacache_t* h, int32_t B, const void* q_
                       map_output(o.cand_prefix_scores, &dev.cand_prefix_scores);
   if (!mapped) return LACACHE_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
+  if (reads_host_inputs(h, B, src[0], src[1], src[2]))
+    return run_lookup(h, B, src[0], src[1], static_cast<const int32_t*>(src[2]), dev, st, Inputs::kHost);
   next_stage_slot(h);
   if (launch_gather(h, g, gathered, st) != cudaSuccess) return LACACHE_ERR_CUDA;
-  return run_lookup(h, B, in.dst[0], in.dst[1], reinterpret_cast<const int32_t*>(in.dst[2]), dev, st, true);
+  return run_lookup(h, B, in.dst[0], in.dst[1], reinterpret_cast<const int32_t*>(in.dst[2]), dev, st,
+                    Inputs::kGathered);
 }
 
 lacache_status lacache_append_misses(lacache_t* h, int32_t B, const void* q_emb_dev, const void* q_prefix_dev,

@@ -92,6 +92,7 @@ struct Stage1Args {
                               // (nullptr: static schedule)
   int inputs_from_previous;   // tensor kernel: the queries are written by the grid launched just before (the
                               // host-input gather), so wait for it before reading anything
+  int q_host;                 // streaming kernel: q is mapped host memory
 };
 
 struct Stage2Args {
@@ -114,6 +115,7 @@ struct Stage2Args {
   const int32_t* q_ids;          // [B x k]
   lacache_result out;            // device pointers
   unsigned long long* counters;  // decision counters [hits, rejects, key misses], or nullptr
+  int host_inputs;               // the query inputs lie in mapped host memory
 };
 
 // cuTensorMapEncodeTiled, obtained from the driver at run time.

@@ -50,6 +50,7 @@ struct StreamParams {
   uint64_t* part_cand;
   PartMeta* part_meta;
   int wait_first;     // the queries are written by the grid launched just before: wait before reading them
+  int q_host;         // the queries lie in mapped host memory
 };
 
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
@@ -115,31 +116,6 @@ __global__ void __launch_bounds__(kThreads, 1) stage1_stream_kernel(const Stream
   float* best = thr + kWarps * qpad;                                              // [kWarps][qpad]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  // Launched as a programmatic dependent of the previous grid on the stream (the previous lookup's stage 2, which
-  // reads the partial lists this grid writes and writes nothing it reads): the scan runs alongside it, and every
-  // thread waits for it only before writing the partial lists. When the queries come from the grid just before
-  // (the host-input gather), every thread waits here instead, before reading them.
-  if (p.wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-  for (int i = threadIdx.x; i < qpad * dc; i += kThreads) {
-    const int r = i / dc, c = i - r * dc;
-    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-    if (r < p.qn) {
-      const uint4 v = load_chunk(p.q + (int64_t)(p.q0 + r) * p.d, c);
-      lo = make_float4(bf_lo(v.x), bf_hi(v.x), bf_lo(v.y), bf_hi(v.y));
-      hi = make_float4(bf_lo(v.z), bf_hi(v.z), bf_lo(v.w), bf_hi(v.w));
-    }
-    qlo[i] = lo;
-    qhi[i] = hi;
-  }
-  for (int i = threadIdx.x; i < kWarps * qpad * C; i += kThreads) lists[i] = 0;
-  for (int i = threadIdx.x; i < kWarps * qpad; i += kThreads) {
-    thr[i] = p.tau_c;
-    best[i] = -INFINITY;
-  }
-  __syncthreads();
-
   constexpr int V = KT * QB;           // scores per tile and query group
   constexpr int SPREAD = 32 / V;       // lanes that end the reduction with the same score
   constexpr int QS = QB < 4 ? QB : 4;  // queries whose chunk values sit in registers at once
@@ -153,88 +129,144 @@ __global__ void __launch_bounds__(kThreads, 1) stage1_stream_kernel(const Stream
   const int groups = qpad / QB;
 
   // one warp tile: keys [t0, t0 + KT), those at or past j_end absent
-  auto tile = [&](int64_t t0, int64_t j_end) {
-    for (int g = 0; g < groups; ++g) {
-      float2 acc[KT][QB];
+  uint4 kv[KT][PH];
+  // a phase's chunks of the tile's keys, all loads in flight together
+  auto load_phase = [&](int64_t t0, int64_t j_end, int ph) {
 #pragma unroll
-      for (int kt = 0; kt < KT; ++kt)
+    for (int kt = 0; kt < KT; ++kt) {
+      const int64_t j = t0 + kt;
+      const __nv_bfloat16* row = p.keys + j * p.d;
 #pragma unroll
-        for (int q = 0; q < QB; ++q) acc[kt][q] = make_float2(0.f, 0.f);
-      for (int ph = 0; ph < p.nph; ++ph) {
-        uint4 kv[KT][PH];
+      for (int i = 0; i < PH; ++i) {
+        const int c = (ph * PH + i) * 32 + lane;
+        kv[kt][i] = (j < j_end && c < dc) ? load_chunk(row, c) : make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+  };
+  float2 acc[KT][QB];
+  auto clear = [&]() {
+#pragma unroll
+    for (int kt = 0; kt < KT; ++kt)
+#pragma unroll
+      for (int q = 0; q < QB; ++q) acc[kt][q] = make_float2(0.f, 0.f);
+  };
+  auto add_phase = [&](int g, int ph) {
+#pragma unroll
+    for (int i = 0; i < PH; ++i) {
+      const int c = (ph * PH + i) * 32 + lane;
+      if (c >= dc) continue;
+#pragma unroll
+      for (int qs = 0; qs < QB; qs += QS) {
+        float2 qv[QS][4];
+#pragma unroll
+        for (int q = 0; q < QS; ++q) {
+          const float4 a = qlo[(size_t)(g * QB + qs + q) * dc + c];
+          const float4 b = qhi[(size_t)(g * QB + qs + q) * dc + c];
+          qv[q][0] = make_float2(a.x, a.y);
+          qv[q][1] = make_float2(a.z, a.w);
+          qv[q][2] = make_float2(b.x, b.y);
+          qv[q][3] = make_float2(b.z, b.w);
+        }
 #pragma unroll
         for (int kt = 0; kt < KT; ++kt) {
-          const int64_t j = t0 + kt;
-          const __nv_bfloat16* row = p.keys + j * p.d;
+          const uint4 w = kv[kt][i];
+          const float2 k0 = make_float2(bf_lo(w.x), bf_hi(w.x)), k1 = make_float2(bf_lo(w.y), bf_hi(w.y));
+          const float2 k2 = make_float2(bf_lo(w.z), bf_hi(w.z)), k3 = make_float2(bf_lo(w.w), bf_hi(w.w));
 #pragma unroll
-          for (int i = 0; i < PH; ++i) {
-            const int c = (ph * PH + i) * 32 + lane;
-            kv[kt][i] = (j < j_end && c < dc) ? load_chunk(row, c) : make_uint4(0u, 0u, 0u, 0u);
-          }
-        }
-#pragma unroll
-        for (int i = 0; i < PH; ++i) {
-          const int c = (ph * PH + i) * 32 + lane;
-          if (c >= dc) continue;
-#pragma unroll
-          for (int qs = 0; qs < QB; qs += QS) {
-            float2 qv[QS][4];
-#pragma unroll
-            for (int q = 0; q < QS; ++q) {
-              const float4 a = qlo[(size_t)(g * QB + qs + q) * dc + c];
-              const float4 b = qhi[(size_t)(g * QB + qs + q) * dc + c];
-              qv[q][0] = make_float2(a.x, a.y);
-              qv[q][1] = make_float2(a.z, a.w);
-              qv[q][2] = make_float2(b.x, b.y);
-              qv[q][3] = make_float2(b.z, b.w);
-            }
-#pragma unroll
-            for (int kt = 0; kt < KT; ++kt) {
-              const uint4 w = kv[kt][i];
-              const float2 k0 = make_float2(bf_lo(w.x), bf_hi(w.x)), k1 = make_float2(bf_lo(w.y), bf_hi(w.y));
-              const float2 k2 = make_float2(bf_lo(w.z), bf_hi(w.z)), k3 = make_float2(bf_lo(w.w), bf_hi(w.w));
-#pragma unroll
-              for (int q = 0; q < QS; ++q) {
-                float2 t = acc[kt][qs + q];
-                t = ffma2(k0, qv[q][0], t);
-                t = ffma2(k1, qv[q][1], t);
-                t = ffma2(k2, qv[q][2], t);
-                t = ffma2(k3, qv[q][3], t);
-                acc[kt][qs + q] = t;
-              }
-            }
+          for (int q = 0; q < QS; ++q) {
+            float2 t = acc[kt][qs + q];
+            t = ffma2(k0, qv[q][0], t);
+            t = ffma2(k1, qv[q][1], t);
+            t = ffma2(k2, qv[q][2], t);
+            t = ffma2(k3, qv[q][3], t);
+            acc[kt][qs + q] = t;
           }
         }
       }
-      // threshold, best score and top_c of the tile's scores for query group g
-      float x[V];
+    }
+  };
+  // threshold, best score and top_c of the tile's scores for query group g
+  auto finish = [&](int64_t t0, int64_t j_end, int g) {
+    float x[V];
 #pragma unroll
-      for (int kt = 0; kt < KT; ++kt)
+    for (int kt = 0; kt < KT; ++kt)
 #pragma unroll
-        for (int q = 0; q < QB; ++q) x[kt * QB + q] = acc[kt][q].x + acc[kt][q].y;
-      const float s = reduce_scatter<V>(x, lane);
-      const int gq = g * QB + my_q;
-      const int64_t j = t0 + my_kt;
-      const bool valid = j < j_end && gq < p.qn;
-      float m = valid ? s : -INFINITY;
+      for (int q = 0; q < QB; ++q) x[kt * QB + q] = acc[kt][q].x + acc[kt][q].y;
+    const float s = reduce_scatter<V>(x, lane);
+    const int gq = g * QB + my_q;
+    const int64_t j = t0 + my_kt;
+    const bool valid = j < j_end && gq < p.qn;
+    float m = valid ? s : -INFINITY;
 #pragma unroll
-      for (int o = SPREAD * QB; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (my_kt == 0 && reporter && gq < p.qn && m > my_best[gq]) my_best[gq] = m;
-      const bool cand = valid && reporter && s >= my_thr[gq];
-      unsigned mask = __ballot_sync(0xffffffffu, cand);
-      while (mask) {
-        const int src = __ffs(mask) - 1;
-        mask &= mask - 1;
-        if (lane == src)
-          list_insert(my_lists + (size_t)gq * C, C, pack_cand(s, (uint32_t)j), my_thr + gq, p.tau_c);
-        __syncwarp();
-      }
+    for (int o = SPREAD * QB; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (my_kt == 0 && reporter && gq < p.qn && m > my_best[gq]) my_best[gq] = m;
+    const bool cand = valid && reporter && s >= my_thr[gq];
+    unsigned mask = __ballot_sync(0xffffffffu, cand);
+    while (mask) {
+      const int src = __ffs(mask) - 1;
+      mask &= mask - 1;
+      if (lane == src)
+        list_insert(my_lists + (size_t)gq * C, C, pack_cand(s, (uint32_t)j), my_thr + gq, p.tau_c);
+      __syncwarp();
     }
   };
 
   // the CTA's contiguous split of the keys, its warps interleaved over it
   const int64_t j_begin = p.n * blockIdx.x / p.splits, j_end = p.n * (blockIdx.x + 1) / p.splits;
-  for (int64_t t0 = j_begin + (int64_t)warp * KT; t0 < j_end; t0 += (int64_t)kWarps * KT) tile(t0, j_end);
+  constexpr int64_t kStep = (int64_t)kWarps * KT;
+  int64_t t0 = j_begin + (int64_t)warp * KT;
+  // One query group and one load phase (a row of up to 1024 elements): each tile's loads are issued before the one
+  // before is reduced, and the first tile's before the queries are there.
+  const bool ahead = groups == 1 && p.nph == 1;
+  if (ahead) load_phase(t0, j_end, 0);
+
+  // Launched as a programmatic dependent of the previous grid on the stream (the previous lookup's stage 2, which
+  // reads the partial lists this grid writes and writes nothing it reads): the scan runs alongside it, and every
+  // thread waits for it only before writing the partial lists. When the queries come from the grid just before
+  // (the host-input gather), every thread waits here instead, before reading them.
+  if (p.wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+  for (int i = threadIdx.x; i < qpad * dc; i += kThreads) {
+    const int r = i / dc, c = i - r * dc;
+    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+    if (r < p.qn) {
+      const uint4* src = reinterpret_cast<const uint4*>(p.q + (int64_t)(p.q0 + r) * p.d) + c;
+      // host memory past the caches: the host may have written it since an earlier grid read it
+      const uint4 v = p.q_host ? __ldcv(src) : __ldg(src);
+      lo = make_float4(bf_lo(v.x), bf_hi(v.x), bf_lo(v.y), bf_hi(v.y));
+      hi = make_float4(bf_lo(v.z), bf_hi(v.z), bf_lo(v.w), bf_hi(v.w));
+    }
+    qlo[i] = lo;
+    qhi[i] = hi;
+  }
+  for (int i = threadIdx.x; i < kWarps * qpad * C; i += kThreads) lists[i] = 0;
+  for (int i = threadIdx.x; i < kWarps * qpad; i += kThreads) {
+    thr[i] = p.tau_c;
+    best[i] = -INFINITY;
+  }
+  __syncthreads();
+
+  if (ahead) {
+    while (t0 < j_end) {
+      clear();
+      add_phase(0, 0);
+      const int64_t t = t0;
+      t0 += kStep;
+      load_phase(t0, j_end, 0);
+      finish(t, j_end, 0);
+    }
+  } else {
+    for (; t0 < j_end; t0 += kStep)
+      for (int g = 0; g < groups; ++g) {
+        clear();
+        for (int ph = 0; ph < p.nph; ++ph) {
+          load_phase(t0, j_end, ph);
+          add_phase(g, ph);
+        }
+        finish(t0, j_end, g);
+      }
+  }
 
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -345,6 +377,7 @@ cudaError_t launch_stage1_stream(const Stage1Args& a, int num_sms, int max_split
     p.qn = a.B - q0 < qc ? a.B - q0 : qc;
     p.qpad = (p.qn + qb - 1) / qb * qb;
     p.wait_first = q0 == 0 ? a.inputs_from_previous : 0;
+    p.q_host = a.q_host;
     const cudaError_t e = launch_shape(p, qb, st);
     if (e != cudaSuccess) return e;
   }

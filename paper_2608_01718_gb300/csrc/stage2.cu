@@ -1,6 +1,6 @@
 // Candidate merge, stage 2 (the lookahead check) and the decision, fused in one kernel.
 //
-// One CTA (8 warps) per query:
+// One CTA per query (8 warps; 4 in large batches, see launch_warps):
 //  1. merge the stage-1 partial lists (per split a record of its best score and candidate count, and that many
 //     packed candidates) into C_q, the top_c candidates by (key score desc, entry id asc): every thread keeps a
 //     sorted top-c of the candidates it reads (four splits in flight), each warp reduces its lanes' lists by top_c
@@ -15,8 +15,6 @@
 namespace lc {
 namespace {
 
-constexpr int kWarps = 8;
-constexpr int kThreads = kWarps * 32;
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -62,8 +60,14 @@ __device__ __forceinline__ void keep(uint64_t (&loc)[CPAD], uint64_t x) {
   }
 }
 
-template <int CPAD>
-__global__ void __launch_bounds__(kThreads) stage2_kernel(Stage2Args a) {
+// kHost: the query inputs lie in mapped host memory (a lookup that reads them in place). They go to shared memory, requested
+// before the wait for the grids ahead, and past the caches: the host may have written them since an earlier grid read
+// them.
+template <int CPAD, int kWarps, bool kHost>
+__global__ void __launch_bounds__(kWarps * 32, (kWarps == 8 ? 1 : 2) * (CPAD <= 8 ? 4 : CPAD <= 16 ? 3 : 2))
+    stage2_kernel(Stage2Args a) {
+  constexpr int kThreads = kWarps * 32;
+  extern __shared__ uint4 smem_q[];             // kHost: the query's prefix row [pd bf16], then its token ids [k]
   __shared__ uint64_t warp_top[kWarps][CPAD];
   __shared__ uint64_t cand[CPAD];
   __shared__ float cand_rm[CPAD][kMaxModels];   // every model's r per candidate
@@ -76,6 +80,18 @@ __global__ void __launch_bounds__(kThreads) stage2_kernel(Stage2Args a) {
   const int q = blockIdx.x;
   const int C = a.top_c;
 
+  const int pd = a.pd, k = a.k;
+  const uint4* pq = reinterpret_cast<const uint4*>(a.q_prefix + (int64_t)q * pd);
+  const int32_t* tq = a.q_ids + (int64_t)q * k;
+  if constexpr (kHost) {
+    int32_t* ts = reinterpret_cast<int32_t*>(smem_q + pd / 8);
+    for (int i = threadIdx.x; i < pd / 8; i += kThreads) smem_q[i] = __ldcv(pq + i);
+    for (int i = threadIdx.x; i < k; i += kThreads) ts[i] = __ldcv(tq + i);
+    pq = smem_q;
+    tq = ts;
+  }
+  auto query16 = [&](int i) { return kHost ? pq[i] : __ldg(pq + i); };
+  auto token = [&](int i) { return kHost ? tq[i] : __ldg(tq + i); };
   // Launched as a programmatic dependent of stage 1: wait until every preceding grid on the stream has completed
   // and its writes are visible, before reading anything (a no-op when launched without the attribute).
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -160,27 +176,24 @@ __global__ void __launch_bounds__(kThreads) stage2_kernel(Stage2Args a) {
   const int n_cand = s_ncand;
 
   // 2. lookahead check of every candidate, one warp per candidate; one dot product per model segment
-  const int pd = a.pd, k = a.k;
-  const uint4* pq = reinterpret_cast<const uint4*>(a.q_prefix + (int64_t)q * pd);
-  const int32_t* tq = a.q_ids + (int64_t)q * k;
   for (int i = warp; i < n_cand; i += kWarps) {
     const uint32_t j = cand_id(cand[i]);
     const uint4* pj = reinterpret_cast<const uint4*>(a.prefix + (int64_t)j * pd);
     const int32_t* tj = a.ids + (int64_t)j * k;
     // the first 32 token ids of both prefixes, loaded with the prefix rows below rather than after them
     const bool tl = lane < k;
-    const int32_t tq0 = tl ? __ldg(tq + lane) : 0, tj0 = tl ? __ldg(tj + lane) : 0;
+    const int32_t tq0 = tl ? token(lane) : 0, tj0 = tl ? __ldg(tj + lane) : 0;
     int emb_ok = 1;
     for (int h = 0; h < a.m; ++h) {
       float acc = 0.f;
       for (int c8 = a.seg[h] / 8 + lane; c8 < a.seg[h + 1] / 8; c8 += 32)
-        acc = dot8(__ldg(pq + c8), __ldg(pj + c8), acc);
+        acc = dot8(query16(c8), __ldg(pj + c8), acc);
       const float r = warp_sum(acc);
       emb_ok &= r >= a.tau_m[h] ? 1 : 0;
       if (lane == 0) cand_rm[i][h] = r;
     }
     int eq = tl && tq0 == tj0 ? 1 : 0;
-    for (int t = lane + 32; t < k; t += 32) eq += (__ldg(tq + t) == __ldg(tj + t)) ? 1 : 0;
+    for (int t = lane + 32; t < k; t += 32) eq += (token(t) == __ldg(tj + t)) ? 1 : 0;
     const int m = __reduce_add_sync(kFull, eq);
     if (lane == 0) {
       cand_emb_ok[i] = emb_ok;
@@ -241,31 +254,43 @@ __global__ void __launch_bounds__(kThreads) stage2_kernel(Stage2Args a) {
 
 // Programmatic dependent launch: the grid may be scheduled while stage 1 is still running (its CTAs then sit in
 // griddepcontrol.wait), which hides the launch gap between the two kernels.
-template <int CPAD>
+template <int CPAD, int kWarps, bool kHost>
 cudaError_t launch_cpad(const Stage2Args& a, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.B);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = 0;
+  cfg.blockDim = dim3(kWarps * 32);
+  cfg.dynamicSmemBytes = kHost ? (size_t)a.pd * 2 + (size_t)a.k * 4 : 0;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, stage2_kernel<CPAD>, a);
+  return cudaLaunchKernelEx(&cfg, stage2_kernel<CPAD, kWarps, kHost>, a);
+}
+
+// Warps per query. The work of a query is a chain of latencies, and eight warps make it shortest; once the queries fill
+// the GPU several times over, the number of them in flight counts instead, and CTAs of four warps hold more. Measured
+// alone (us, eight / four warps): 262,144 entries, top_c = 8, 512 queries 13.8 / 15.8, 1,024 19.3 / 16.9, 8,192 90 / 66;
+// 1M entries, top_c = 16, 512 queries 22.9 / 26.5, 1,024 35.9 / 31.9, 8,192 230 / 195 (295 with 87 registers a thread).
+constexpr int kLargeBatch = 1024;
+
+template <int CPAD>
+cudaError_t launch_warps(const Stage2Args& a, cudaStream_t st) {
+  if (a.host_inputs) return launch_cpad<CPAD, 8, true>(a, st);
+  return a.B >= kLargeBatch ? launch_cpad<CPAD, 4, false>(a, st) : launch_cpad<CPAD, 8, false>(a, st);
 }
 
 cudaError_t launch_stage2(const Stage2Args& a, cudaStream_t st) {
   cudaError_t e;
   if (a.top_c <= 4)
-    e = launch_cpad<4>(a, st);
+    e = launch_warps<4>(a, st);
   else if (a.top_c <= 8)
-    e = launch_cpad<8>(a, st);
+    e = launch_warps<8>(a, st);
   else if (a.top_c <= 16)
-    e = launch_cpad<16>(a, st);
+    e = launch_warps<16>(a, st);
   else
-    e = launch_cpad<32>(a, st);
+    e = launch_warps<32>(a, st);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

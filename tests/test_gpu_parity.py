@@ -600,3 +600,32 @@ def test_append_takes_the_non_hit_rows_in_query_order(B):
             L.lacache_read_rows(cache.h, n0, m, key, prefix, tok)
             cache.sync()
             assert torch.equal(key, emb[miss]) and torch.equal(prefix, pre[miss]) and torch.equal(tok, ids[miss])
+
+
+@pytest.mark.parametrize("d,batch", [(768, 1), (768, 4), (768, 5), (1024, 3), (1280, 2), (392, 7)])
+def test_host_lookups_read_small_batches_in_place(d, batch):
+    # streaming-scan lookups from mapped pinned memory: batches of at most 1 MiB over all SMs (4 queries at d = 768, 3 at
+    # 1024, 8 at 392) are read where they are, others gathered first. The same buffers are refilled between calls, so a
+    # stale cache line would show; three lookups are in flight in the asynchronous form.
+    w = wl.WORKLOADS["mid-1m"].scaled(n=9_000, d=d, batch=batch, clusters=90)
+    with new_cache(w, L.LACACHE_STAGE1_STREAM) as cache:
+        fill(cache, w)
+        qs = [wl.batch(w, i, device="cuda") for i in range(3)]
+        want = [gpu_lookup(cache, q) for q in qs]
+        host = {k: torch.empty_like(qs[0][k], device="cpu").pin_memory() for k in ("emb", "prefix", "ids")}
+        out = L.alloc_result(w.batch, w.top_c, "cpu", pinned=True)
+        for q, g in zip(qs, want):
+            for k, v in host.items():
+                v.copy_(q[k])
+            L.lacache_lookup_host(cache.h, host["emb"], host["prefix"], host["ids"], out)
+            for k, v in out.items():
+                assert np.array_equal(v.numpy(), g[k], equal_nan=True), k
+        hq = [{k: q[k].cpu().pin_memory() for k in host} for q in qs]
+        outs = [L.alloc_result(w.batch, w.top_c, "cpu", pinned=True) for _ in qs]
+        stream = torch.cuda.current_stream()
+        for q, o in zip(hq, outs):
+            L.lacache_lookup_host_async(cache.h, q["emb"], q["prefix"], q["ids"], o, stream)
+        stream.synchronize()
+        for o, g in zip(outs, want):
+            for k, v in o.items():
+                assert np.array_equal(v.numpy(), g[k], equal_nan=True), k
