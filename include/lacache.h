@@ -60,8 +60,8 @@ typedef enum { LACACHE_BF16 = 0, LACACHE_F32 = 1 } lacache_dtype;
 
 /* Which stage-1 kernel lookups run. */
 typedef enum {
-  LACACHE_STAGE1_AUTO = 0,   /* the streaming scan when n x d x B <= 2^25 (few enough multiply-adds that its
-                                latency is the shorter: at most 64 MiB of keys at one query) and for 1 or 2
+  LACACHE_STAGE1_AUTO = 0,   /* the streaming scan for up to 24 queries when n x d x B <= 2^25 (few enough
+                                multiply-adds: at most 64 MiB of keys at one query) and for 1 or 2
                                 queries at d = 1024 (where it matches the tensor-core scan from HBM); the
                                 tensor-core scan otherwise, which holds the HBM roofline at every batch size */
   LACACHE_STAGE1_TENSOR = 1, /* tcgen05 tensor-core scan (TMA-fed, TMEM accumulators) */

@@ -180,10 +180,14 @@ inline int lsh_tensor_min_batch(int bits) { return bits == 256 ? 48 : 40; }
 // 13.3, B = 2: 13.6 against 13.1. A single lookup on an idle device crosses later (16,384 x 768, B = 4: 18.2
 // against 21.2 us), and from a flushed L2 the streaming scan's stage 1 is also the shorter one at that size (22.3
 // against 25.9 us at 43,690 x 768, B = 1). So the streaming scan takes the lookups with n d B <= 2^25 (at most
-// 64 MiB of keys, at one query).
+// 64 MiB of keys, at one query). Since the tensor-core scan takes such stores in tiles of 64 or 128 keys, it is level with
+// the streaming scan at 4 to 16 queries (4,096 x 384, stream / tensor: B = 4 7.5 / 7.1, B = 16 8.5 / 7.1) and well ahead
+// beyond (1,000 x 384: B = 32 13.8 / 8.3, B = 64 23.4 / 8.4; 4,096 x 128: B = 64 15.3 / 7.2), so batches of more than 24
+// queries, three of the streaming scan's query groups, go to it whatever their size.
 constexpr int64_t kStreamAutoMacs = (int64_t)1 << 25;
+constexpr int kStreamAutoBatch = 24;
 inline int auto_stage1(int64_t n, int d, int B) {
-  if (n * d * B <= kStreamAutoMacs) return LACACHE_STAGE1_STREAM;
+  if (B <= kStreamAutoBatch && n * d * B <= kStreamAutoMacs) return LACACHE_STAGE1_STREAM;
   if (B <= 2 && d == 1024) return LACACHE_STAGE1_STREAM;
   return LACACHE_STAGE1_TENSOR;
 }

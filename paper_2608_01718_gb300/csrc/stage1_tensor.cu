@@ -38,10 +38,9 @@ namespace lc {
 namespace {
 
 constexpr int BM = 128;                     // queries per tile (TMEM lanes)
-constexpr int BN = 256;                     // keys per tile (accumulator columns)
+constexpr int kBN = 256;                    // keys per tile (accumulator columns)
 constexpr int BK = 64;                      // bf16 per k-step = one 128-byte swizzled row
 constexpr int A_BYTES = BM * BK * 2;        // 16 KB
-constexpr int TMEM_COLS = 2 * BN;           // two accumulators
 constexpr int kThreads = 192;
 constexpr int kEpiWarps = 4;
 constexpr int RING = 4;                             // tile-index ring of the dynamic schedule
@@ -49,11 +48,12 @@ constexpr size_t kStashBytes = 32 * 129 * 4;          // epilogue's rare-path ch
 constexpr int kMaxDeviceSlots = 64;                   // devices whose CTA-pair capacity is cached
 constexpr int64_t kPairSplitBytes = (int64_t)11 << 20;  // keys per split of the CTA-pair schedule (L2 reuse)
 
-// Per-CTA geometry. Single CTA: the whole 256-key box per stage, 4 stages. CTA pair: half the key box, so 6
-// stages fit in the same shared memory.
-template <bool PAIR>
+// Per-CTA geometry. Single CTA: the whole key box per stage, 4 stages of 256 keys (6 of 128, 8 of 64, on small stores: see
+// tile_keys). CTA pair: half the key box, so 6 stages fit in the same shared memory.
+template <bool PAIR, int BN>
 struct Geo {
-  static constexpr int kStages = PAIR ? 6 : 4;
+  static constexpr int kStages = PAIR || BN == 128 ? 6 : BN == 64 ? 8 : 4;
+  static constexpr int kTmemCols = 2 * BN;                 // two accumulators
   static constexpr int kBRows = PAIR ? BN / 2 : BN;        // key rows this CTA loads per tile
   static constexpr int kBBytes = kBRows * BK * 2;
   static constexpr int kStageBytes = A_BYTES + kBBytes;
@@ -65,7 +65,9 @@ struct Geo {
   static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                                      ((uint32_t)((PAIR ? 2 * BM : BM) >> 4) << 24);
 };
-static_assert(Geo<false>::kSmem <= 227 * 1024 && Geo<true>::kSmem <= 227 * 1024, "shared memory budget");
+static_assert(Geo<false, kBN>::kSmem <= 227 * 1024 && Geo<true, kBN>::kSmem <= 227 * 1024 &&
+                  Geo<false, 128>::kSmem <= 227 * 1024 && Geo<false, 64>::kSmem <= 227 * 1024,
+              "shared memory budget");
 
 struct TcParams {
   int64_t n;
@@ -136,21 +138,21 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
-template <bool PAIR>
+template <bool PAIR, int BN>
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t accumulate) {
   if constexpr (PAIR)
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(Geo<true>::kIdesc), "r"(accumulate)
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(Geo<true, BN>::kIdesc), "r"(accumulate)
         : "memory");
   else
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(Geo<false>::kIdesc), "r"(accumulate)
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(Geo<false, BN>::kIdesc), "r"(accumulate)
         : "memory");
 }
 // Running top_c of one query: scores descending; among equal scores the earlier (lower) id first, which holds
@@ -199,11 +201,11 @@ struct TopC {
 // in place of the queries, and an epilogue that writes SimHash signatures: bit h of row j's signature is set iff
 // <r_h, row_j> >= 0; each warp's 32 hyperplanes form one 32-bit word, packed with a ballot per key column.
 // PAIR = true: launched as two-CTA clusters, static schedule over (query-tile pair, split) units.
-template <int CPAD, bool SIGN, bool PAIR>
+template <int CPAD, bool SIGN, bool PAIR, int BN>
 __global__ void __launch_bounds__(kThreads, 1)
     stage1_tensor_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_l,
                          const __grid_constant__ CUtensorMap tmap_k, const TcParams p) {
-  using G = Geo<PAIR>;
+  using G = Geo<PAIR, BN>;
   constexpr int S = G::kStages;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -255,7 +257,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // shared memory or allocates the pair's TMEM.
   if constexpr (PAIR) cluster_sync();
   if (warp == 1) {
-    tmem_alloc<PAIR>(smem_u32(tmem_slot), TMEM_COLS);
+    tmem_alloc<PAIR>(smem_u32(tmem_slot), G::kTmemCols);
     tmem_relinquish<PAIR>();
   }
   tc_fence_before();
@@ -404,7 +406,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
               if (kk < n_mma)
-                mma_bf16<PAIR>(d_tmem, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), (ks | kk) != 0 ? 1u : 0u);
+                mma_bf16<PAIR, BN>(d_tmem, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), (ks | kk) != 0 ? 1u : 0u);
             mma_commit<PAIR>(empty_bar(s), 3);
             if (ks + 1 == p.k_steps) mma_commit<PAIR>(tfull_bar(b), 3);
           }
@@ -587,7 +589,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if constexpr (PAIR) cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc<PAIR>(tmem, TMEM_COLS);
+    tmem_dealloc<PAIR>(tmem, G::kTmemCols);
   }
 }
 
@@ -604,12 +606,12 @@ struct Maps {
   CUtensorMap q, last, k;   // query tile, last query tile, key tile
 };
 
-template <int CPAD, bool SIGN, bool PAIR>
+template <int CPAD, bool SIGN, bool PAIR, int BN>
 cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = Geo<PAIR>::kSmem;
+  cfg.dynamicSmemBytes = Geo<PAIR, BN>::kSmem;
   cfg.stream = st;
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -622,14 +624,14 @@ cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, cudaS
   return cfg;
 }
 
-template <int CPAD, bool SIGN, bool PAIR>
+template <int CPAD, bool SIGN, bool PAIR, int BN>
 cudaError_t launch_cpad(const Maps& m, const TcParams& p, int grid, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(stage1_tensor_kernel<CPAD, SIGN, PAIR>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<PAIR>::kSmem);
+  cudaError_t e = cudaFuncSetAttribute(stage1_tensor_kernel<CPAD, SIGN, PAIR, BN>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<PAIR, BN>::kSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[2];
-  cudaLaunchConfig_t cfg = launch_config<CPAD, SIGN, PAIR>(attr, grid, st);
-  e = cudaLaunchKernelEx(&cfg, stage1_tensor_kernel<CPAD, SIGN, PAIR>, m.q, m.last, m.k, p);
+  cudaLaunchConfig_t cfg = launch_config<CPAD, SIGN, PAIR, BN>(attr, grid, st);
+  e = cudaLaunchKernelEx(&cfg, stage1_tensor_kernel<CPAD, SIGN, PAIR, BN>, m.q, m.last, m.k, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -637,15 +639,15 @@ cudaError_t launch_cpad(const Maps& m, const TcParams& p, int grid, cudaStream_t
 // CTA pairs of this kernel that can be resident at once on the current device (0: none, or not supported).
 template <int CPAD>
 int max_pair_clusters(cudaStream_t st) {
-  if (cudaFuncSetAttribute(stage1_tensor_kernel<CPAD, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)Geo<true>::kSmem) != cudaSuccess) {
+  if (cudaFuncSetAttribute(stage1_tensor_kernel<CPAD, false, true, kBN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)Geo<true, kBN>::kSmem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   cudaLaunchAttribute attr[2];
-  cudaLaunchConfig_t cfg = launch_config<CPAD, false, true>(attr, 2, st);
+  cudaLaunchConfig_t cfg = launch_config<CPAD, false, true, kBN>(attr, 2, st);
   int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, stage1_tensor_kernel<CPAD, false, true>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&clusters, stage1_tensor_kernel<CPAD, false, true, kBN>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -701,7 +703,7 @@ bool launch_pairs(TcParams p, const Stage1Args& a, EncodeTiledFn encode, int max
   if (clusters < 1) return false;
   p.pairs = (p.q_tiles + 1) / 2;
   Maps m;
-  if (!encode_maps(encode, &m, p, a.q, a.B, a.keys, a.n, (uint32_t)Geo<true>::kBRows)) {
+  if (!encode_maps(encode, &m, p, a.q, a.B, a.keys, a.n, (uint32_t)Geo<true, kBN>::kBRows)) {
     *err = cudaErrorInvalidValue;
     return true;
   }
@@ -724,7 +726,7 @@ bool launch_pairs(TcParams p, const Stage1Args& a, EncodeTiledFn encode, int max
   p.units = p.pairs * s;
   *splits = s;
   const int grid = 2 * (p.units < clusters ? p.units : clusters);
-  *err = launch_cpad<CPAD, false, true>(m, p, grid, st);
+  *err = launch_cpad<CPAD, false, true, kBN>(m, p, grid, st);
   return true;
 }
 
@@ -739,6 +741,17 @@ bool use_pairs(int q_tiles, int d, int64_t n_tiles, int num_sms) {
   return !(q_tiles % 2 == 1 && q_tiles <= 5 && d % 128 == 0 && n_tiles >= 4 * (int64_t)num_sms);
 }
 
+// Keys per tile of a scan of q_tiles query tiles: 64 or 128 for one query tile on a store that gives no SM more than one
+// such tile. The scan is then a chain of latencies (set-up, one tile's loads, MMAs, epilogue and insertions), shorter for a
+// smaller tile, and 256-key tiles would leave most SMs idle. From two tiles per SM on, the 256-key tile's longer loads win.
+// Measured (us a lookup, 64 queries, 256-key tiles / these): 300 x 384 19.3 / 10.3, 1,000 x 384 16.3 / 8.4, 4,096 x 384
+// 11.0 / 7.4, 9,700 x 768 11.9 / 8.6, 9,800 x 768 11.6 / 9.6, 19,000 x 768 11.3 / 9.8; two tiles: 20,000 x 768 in 64-key
+// tiles 11.5 / 14.4, 19,500 x 768 in 128-key tiles 11.3 / 11.9.
+int tile_keys(int q_tiles, int64_t n, int num_sms) {
+  if (q_tiles > 1) return kBN;
+  return n <= 64 * (int64_t)num_sms ? 64 : n <= 128 * (int64_t)num_sms ? 128 : kBN;
+}
+
 template <int CPAD>
 cudaError_t launch_key_check(TcParams p, const Stage1Args& a, EncodeTiledFn encode, int num_sms, int max_splits,
                              cudaStream_t st, int* splits, bool* paired) {
@@ -747,8 +760,11 @@ cudaError_t launch_key_check(TcParams p, const Stage1Args& a, EncodeTiledFn enco
     if (paired) *paired = true;
     return err;
   }
+  const int bn = tile_keys(p.q_tiles, a.n, num_sms);
+  p.n_tiles = (a.n + bn - 1) / bn;
   Maps m;
-  if (!encode_maps(encode, &m, p, a.q, a.B, a.keys, a.n, (uint32_t)BN)) return cudaErrorInvalidValue;
+  if (!encode_maps(encode, &m, p, a.q, a.B, a.keys, a.n, (uint32_t)bn))
+    return cudaErrorInvalidValue;
   // splits such that q_tiles * splits is a multiple of the SM count (whole waves of units); one query tile with
   // a tile counter: a dynamic schedule with one split per CTA
   int s = num_sms / gcd_int(num_sms, p.q_tiles);
@@ -760,7 +776,9 @@ cudaError_t launch_key_check(TcParams p, const Stage1Args& a, EncodeTiledFn enco
   if (p.q_tiles == 1 && a.tile_ctr) p.tile_ctr = a.tile_ctr;
   *splits = s;
   const int grid = p.units < num_sms ? p.units : num_sms;
-  return launch_cpad<CPAD, false, false>(m, p, grid, st);
+  return bn == 64    ? launch_cpad<CPAD, false, false, 64>(m, p, grid, st)
+         : bn == 128 ? launch_cpad<CPAD, false, false, 128>(m, p, grid, st)
+                     : launch_cpad<CPAD, false, false, kBN>(m, p, grid, st);
 }
 
 }  // namespace
@@ -778,7 +796,7 @@ cudaError_t launch_signatures(const __nv_bfloat16* rows, int64_t n, int d, const
   p.top_c = 1;
   p.q_tiles = (bits + BM - 1) / BM;
   p.last_rows = (bits - (p.q_tiles - 1) * BM + 7) / 8 * 8;
-  p.n_tiles = (n + BN - 1) / BN;
+  p.n_tiles = (n + kBN - 1) / kBN;
   p.k_steps = (d + BK - 1) / BK;
   p.last_mmas = (d - (p.k_steps - 1) * BK + 15) / 16;
   int s = num_sms / gcd_int(num_sms, p.q_tiles);
@@ -790,9 +808,9 @@ cudaError_t launch_signatures(const __nv_bfloat16* rows, int64_t n, int d, const
   p.sig_words = bits / 32;
   p.dev_status = dev_status;
   Maps m;
-  if (!encode_maps(encode, &m, p, hyperplanes, bits, rows, n, (uint32_t)BN)) return cudaErrorInvalidValue;
+  if (!encode_maps(encode, &m, p, hyperplanes, bits, rows, n, (uint32_t)kBN)) return cudaErrorInvalidValue;
   const int grid = p.units < num_sms ? p.units : num_sms;
-  return launch_cpad<4, true, false>(m, p, grid, st);
+  return launch_cpad<4, true, false, kBN>(m, p, grid, st);
 }
 
 cudaError_t launch_stage1_tensor(const Stage1Args& a, EncodeTiledFn encode, int num_sms, int max_splits,
@@ -806,7 +824,7 @@ cudaError_t launch_stage1_tensor(const Stage1Args& a, EncodeTiledFn encode, int 
   p.top_c = a.top_c;
   p.q_tiles = (a.B + BM - 1) / BM;
   p.last_rows = (a.B - (p.q_tiles - 1) * BM + 7) / 8 * 8;
-  p.n_tiles = (a.n + BN - 1) / BN;
+  p.n_tiles = (a.n + kBN - 1) / kBN;
   p.k_steps = (a.d + BK - 1) / BK;
   p.last_mmas = (a.d - (p.k_steps - 1) * BK + 15) / 16;
   p.part_cand = a.part_cand;

@@ -78,6 +78,24 @@ def test_ragged_batch_dimension_and_k(stage1):
     assert rep.exact + rep.band == w.batch and rep.band <= 2
 
 
+@pytest.mark.parametrize("n", [1, 64, 65, 9_728, 9_729, 19_456, 19_457])
+@pytest.mark.parametrize("batch", [25, 128])
+def test_small_store_tile_sizes(n, batch):
+    # one query tile on a small store: 64-key tiles while no SM gets two (9,728 entries on 152 SMs), then 128-key tiles
+    # (19,456), then 256; a store of one tile, of one key, and a key past each limit. AUTO takes the tensor scan for more
+    # than 24 queries, however small the store.
+    w = wl.WORKLOADS["mid-1m"].scaled(n=n, d=72, batch=batch, clusters=max(1, n // 300))
+    st = oracle_store(w)
+    with new_cache(w, L.LACACHE_STAGE1_AUTO) as cache:
+        fill(cache, w)
+        q = wl.batch(w, 0, device="cuda")
+        g = gpu_lookup(cache, q)
+        assert cache.last_launch()[1] == L.LACACHE_STAGE1_TENSOR
+    oq, p = oracle_queries(q), params(w)
+    rep = compare(g, oracle.lookup(st, oq, p), p, pair_scores=pair_scores_fn(st, oq))
+    assert rep.exact + rep.band == w.batch and rep.band <= w.batch // 10
+
+
 @pytest.mark.parametrize("n,d,batch,pairs", [(5_000, 392, 129, True), (5_000, 136, 250, True), (3_000, 1000, 257, True),
                                              (160_000, 128, 257, False), (160_000, 128, 520, False),
                                              (160_000, 128, 769, True), (160_000, 136, 257, True)])
