@@ -13,15 +13,15 @@
 // per pass into shared memory in the 128-byte swizzle layout.
 //
 // One CTA per contiguous range of 128-entry blocks, warp-specialised:
-//   warp 27 (loader): cp.async.bulk of one stage (8 KB of packed signatures, kBPS blocks) into an 8-deep ring;
-//   warps 22-25 (expanders; warp w writes TMEM lane quadrant w % 4): read their 32 entries' words of a block from the
-//     ring, expand them and store them to one of kABuf A buffers in TMEM;
-//   warp 26 (MMA): allocates TMEM; per block issues tcgen05.mma.kind::f8f6f4 (M = 128 entries, N = the pass's
+//   warp 31 (loader): cp.async.bulk of one stage (8 KB of packed signatures, kBPS blocks) into an 8-deep ring;
+//   warps 22-29 (expanders, two sets of four that take blocks in turn; warp w writes TMEM lane quadrant w % 4): read
+//     their 32 entries' words of a block from the ring, expand them and store them to one of kABuf A buffers in TMEM;
+//   warp 30 (MMA): allocates TMEM; per block issues tcgen05.mma.kind::f8f6f4 (M = 128 entries, N = the pass's
 //     queries rounded up to 32, K = 32) over the resident query operand, into one of up to 8 accumulators;
 //   warps 0-15 (mask warps; warp w reads TMEM lane quadrant w % 4 and the 32-query column chunk w / 4): read each
-//     entry's dot products, and only where their maximum reaches the threshold turn them into a mask of the admitted
-//     queries and queue those (query, entry) pairs in shared memory, each as one word that also holds the queue's
-//     epoch; release the accumulator;
+//     entry's dot products into registers and release the accumulator; only where their maximum reaches the threshold
+//     turn them into a mask of the admitted queries and queue those (query, entry) pairs in shared memory, each as one
+//     word that also holds the queue's epoch;
 //   warps 16-21 (checker warps): claim queued pairs as they arrive, compute their exact fp32 key scores over the
 //     gathered key rows (each lane's 8-element chunks in order, then a butterfly sum) while the scan goes on, and
 //     fold each score into its query's best score and, if it clears tau_c, into the query's list (lock-free). The
@@ -36,15 +36,20 @@
 // CTA records LACACHE_ERR_DEVICE_TIMEOUT in the status word, the roles stop at the next pass boundary, in-flight
 // copies and MMAs are drained, TMEM is freed and the CTA exits.
 //
-// What bounds it: instruction issue and latency in the mask and checker warps, at some 1,700 cycles per block of 128
-// entries at 128 queries and 256 bits; the packed index takes 20 us of HBM time on 4M entries, the MMAs 55 us. Four mask
-// warps share a block's columns, since accumulators for only three blocks fit beside the A buffers; they meet at a
-// barrier only every 32 blocks (every 8: 10 % slower); the roles' loops are rolled, to share the instruction cache.
-// Measured per lookup step against the scan over an index kept expanded in HBM that this one replaces (us, before /
-// after): 4M x 768, 256 bits, 48 queries 177 / 169, 64 180 / 171, 128 202 / 184; 128 bits, 128 queries 184 / 175; 512
-// bits, 64 queries 326 / 219, 128 631 / 238; 1M x 1024, 256 bits, 128 queries 70 / 63, 357 181 / 167; 36,433 x 768, 357
-// queries 44 / 40. (Without the mask warps' help at the end of the range 48 queries on 4M x 768 take 150, but 128 on
-// 4M x 1024 take 233 instead of 198, and 357 on 36,433 x 768 take 49.) The index takes an eighth of the memory, and signing
+// What bounds it: instruction issue (0.67 a scheduler and cycle at 128 queries and 256 bits, ALU pipe half busy), at
+// some 1,500 cycles per block of 128 entries at 128 queries; the packed index takes 20 us of HBM time on 4M entries,
+// the MMAs 55 us. So the warps' loops are kept short, and in 64 registers a thread almost without spills (32-bit entry
+// numbers, no running counts: 8 % at 128 queries); two expander sets, since one took 1,000 cycles a block and the MMAs
+// waited for it (48 queries 166, with two 151); accumulators are released before their scores are looked at, not after
+// the admitted pairs are queued, and mask warps without a query chunk leave them alone (48 queries 145 -> 137). Four
+// mask warps share a block's columns, since accumulators for only three blocks fit beside the A buffers; they meet at a
+// barrier only every 32 blocks (every 16: 2 % slower). Six checker warps: with four, 128 queries take 179 instead of
+// 171; two pairs a checker at a time, or more A buffers, give nothing.
+// Measured per lookup step (us) against the scan over an index kept expanded in HBM that was here first / against one
+// expander set and late release: 4M x 768, 256 bits, 48 queries 177 / 172 -> 128, 64 180 / 175 -> 131, 128 202 / 188 ->
+// 169, 384 -/ 536 -> 477; 128 bits, 48 queries - / 133 -> 116, 128 184 / 163 -> 150; 512 bits, 64 queries 326 / 232 ->
+// 176, 128 631 / 253 -> 222. (Without the mask warps' help at the end of the range 128 queries on 4M x 1024 take 18 %
+// longer, and 357 on 36,433 x 768 a fifth.) The packed index takes an eighth of the expanded one's memory, and signing
 // entries no second kernel.
 #include "internal.cuh"
 #include "tcgen05.cuh"
@@ -56,9 +61,10 @@ constexpr int kMaskParts = 4;                            // mask warps per TMEM 
 constexpr int kMaskWarps = 4 * kMaskParts;               // warps 0-15: lane quadrant w % 4, column chunk w / 4
 constexpr int kCheckWarps = 6;                           // warps 16-21: exact checks of the queued pairs
 constexpr int kEpiWarps = kMaskWarps + kCheckWarps;      // warps 0-21
-constexpr int kExpWarps = 4;                             // warps 22-25: expand entry signatures into TMEM
-constexpr int kMmaWarp = kEpiWarps + kExpWarps;          // warp 26
-constexpr int kLoadWarp = kMmaWarp + 1;                  // warp 27
+constexpr int kExpSets = 2;                              // each takes every second block
+constexpr int kExpWarps = 4 * kExpSets;                  // warps 22-29: expand entry signatures into TMEM
+constexpr int kMmaWarp = kEpiWarps + kExpWarps;          // warp 30
+constexpr int kLoadWarp = kMmaWarp + 1;                  // warp 31
 constexpr int kThreads = (kLoadWarp + 1) * 32;
 constexpr int kCap = 1024;                               // queue capacity
 constexpr int kFlushAt = kCap - kCap / 4;                // a round that leaves more items than this closes the queue
@@ -69,7 +75,7 @@ constexpr int kQC = 128;                                 // queries per pass
 constexpr int kS = 8;                                    // ring stages
 constexpr int kStageBytes = 8192;                        // packed signatures per stage
 constexpr int kMaxNbuf = 8;                              // accumulators (at most)
-constexpr int kABuf = 2;                                 // A buffers
+constexpr int kMaxABuf = 4;                              // A buffers (at most)
 constexpr unsigned kFull = 0xffffffffu;
 
 // Geometry per signature width: W = b / 32 words. TMEM's 512 columns hold kABuf A buffers (128 entries x b bytes, 8 W
@@ -81,13 +87,13 @@ struct TcGeo {
   static constexpr int kBlockBytes = kBlockRows * 4 * W;       // packed: 2, 4 or 8 KB
   static constexpr int kBPS = kStageBytes / kBlockBytes;       // blocks per stage: 4, 2 or 1
   static constexpr int kQueryBytes = kQC * kBits;              // 16, 32 or 64 KB
+  static constexpr int kABuf = W == 4 ? 4 : 2;
   static constexpr int kACols = 8 * W;
   static constexpr int kAccCols = 512 - kABuf * kACols;        // 448, 384 or 256
 };
 constexpr int kChunks = kQC / 32;                        // 32-query chunks of a block (at most)
-constexpr int kOwn = kChunks / kMaskParts;               // ... and of them a mask warp's own
-static_assert(kRound * kOwn <= 32, "a mask thread marks its chunks of a round in one word");
-static_assert(kExpWarps == 4, "an expander warp per TMEM lane quadrant");
+static_assert(kMaskParts == kChunks, "a mask warp has one chunk");
+static_assert(kRound <= 32, "a mask thread marks its blocks of a round in one word");
 static_assert(kEpiWarps * 32 >= 128, "the epilogue threads cover a pass's queries when they set up the lists");
 
 // A queued (query, entry) pair in one word, written and polled as a whole: bits 0-31 the entry id, 32-39 the query within
@@ -110,7 +116,8 @@ struct Tail {
   uint32_t pass_end;           // closed for the last time in the pass
   uint32_t abort_flag;
   uint32_t tmem_slot;
-  uint64_t bars[2 * kS + 2 * kABuf + 2 * kMaxNbuf + 1];   // ring full / empty, A full / empty, accumulator full /
+  uint32_t issued;             // the loader's copies: stages 0 .. issued - 1
+  uint64_t bars[2 * kS + 2 * kMaxABuf + 2 * kMaxNbuf + 1];   // ring full / empty, A full / empty, accumulator full /
                                                              // empty, drain
 };
 
@@ -154,18 +161,23 @@ __device__ __forceinline__ bool mask_any(bool p) {
 }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 2, %0;" ::"n"(kEpiWarps * 32) : "memory"); }
 
-// Maximum of 32 fp32 values given as bits.
+// Maximum of 32 fp32 values given as bits, by the three-operand form (two-operand: 2 % of a lookup at 128 queries).
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
 __device__ __forceinline__ float max32(const uint32_t (&r)[32]) {
-  float m[8];
+  float m[4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
-    m[i] = fmaxf(fmaxf(__uint_as_float(r[i]), __uint_as_float(r[i + 8])),
-                 fmaxf(__uint_as_float(r[i + 16]), __uint_as_float(r[i + 24])));
+  for (int i = 0; i < 4; ++i) {
+    m[i] = __uint_as_float(r[8 * i]);
 #pragma unroll
-  for (int w = 4; w > 0; w >>= 1)
-#pragma unroll
-    for (int i = 0; i < w; ++i) m[i] = fmaxf(m[i], m[i + w]);
-  return m[0];
+    for (int k = 1; k < 7; k += 2)
+      m[i] = max3(m[i], __uint_as_float(r[8 * i + k]), __uint_as_float(r[8 * i + k + 1]));
+    m[i] = fmaxf(m[i], __uint_as_float(r[8 * i + 7]));
+  }
+  return fmaxf(max3(m[0], m[1], m[2]), m[3]);
 }
 
 __device__ __forceinline__ uint32_t ld_volatile(const uint32_t* p) { return *reinterpret_cast<const volatile uint32_t*>(p); }
@@ -217,7 +229,7 @@ __device__ __forceinline__ bool wait_slot(Tail& t, int slot, uint32_t ep, uint64
       atomicOr(dev_status, kDevTimeout);
       return false;
     }
-    __nanosleep(64);
+    __nanosleep(256);
   }
 }
 
@@ -317,27 +329,31 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (kS + s); };
   auto afull_bar = [&](int b) { return bar0 + 8u * (2 * kS + b); };
-  auto aempty_bar = [&](int b) { return bar0 + 8u * (2 * kS + kABuf + b); };
-  auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * kS + 2 * kABuf + b); };
-  auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * kS + 2 * kABuf + kMaxNbuf + b); };
-  const uint32_t drain_bar = bar0 + 8u * (2 * kS + 2 * kABuf + 2 * kMaxNbuf);
+  auto aempty_bar = [&](int b) { return bar0 + 8u * (2 * kS + kMaxABuf + b); };
+  auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * kS + 2 * kMaxABuf + b); };
+  auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * kS + 2 * kMaxABuf + kMaxNbuf + b); };
+  const uint32_t drain_bar = bar0 + 8u * (2 * kS + 2 * kMaxABuf + 2 * kMaxNbuf);
 
   const int warp = __shfl_sync(kFull, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: uniform
+  // accumulators: the same for every pass (the first pass has the most queries). Mask warps of chunks past first_chunks
+  // have none in any pass.
+  const int first_chunks = (min(kQC, a.B) + 31) / 32;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kS; ++s) {
       mbar_init(full_bar(s), 1);              // the loader's arrive, with the copy's bytes
       mbar_init(empty_bar(s), 4 * G::kBPS);   // four expander warps per block of the stage
     }
-    for (int b = 0; b < kABuf; ++b) {
+    for (int b = 0; b < G::kABuf; ++b) {
       mbar_init(afull_bar(b), 4);             // the block's four expander warps
       mbar_init(aempty_bar(b), 1);            // the MMA commit
     }
     for (int b = 0; b < kMaxNbuf; ++b) {
       mbar_init(tfull_bar(b), 1);             // the MMA commit
-      mbar_init(tempty_bar(b), kMaskWarps);
+      mbar_init(tempty_bar(b), 4 * first_chunks);
     }
     mbar_init(drain_bar, 1);
     t.abort_flag = 0;
+    t.issued = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   for (int i = threadIdx.x; i < kCap; i += kThreads) t.items[i] = ~(uint64_t)0;   // no epoch
@@ -360,16 +376,14 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
 
   const int s = blockIdx.x;
   const int64_t nblocks = (a.n + kBlockRows - 1) / kBlockRows;
-  const int64_t g_begin = nblocks * s / splits, g_end = nblocks * (s + 1) / splits;
-  const int64_t j_begin = g_begin * kBlockRows, j_end = min(a.n, g_end * kBlockRows);
-  const uint32_t nb = (uint32_t)(g_end - g_begin);
+  const uint32_t g_begin = (uint32_t)(nblocks * s / splits), nb = (uint32_t)(nblocks * (s + 1) / splits) - g_begin;
+  // the range's entries (ids are int32: so is the store's size)
+  const uint32_t j_begin = g_begin * kBlockRows, j_end = min((uint32_t)a.n, (g_begin + nb) * kBlockRows);
   const uint32_t nstages = (nb + G::kBPS - 1) / G::kBPS;    // ring stages per pass
   const int C = a.top_c;
   const float thr = (float)(G::kBits - 2 * l.radius);   // admitted iff dot >= b - 2 radius
-  // accumulators: the same for every pass (the first pass has the most queries)
-  const int stride = (min(kQC, a.B) + 31) / 32 * 32;
+  const int stride = 32 * first_chunks;
   const uint32_t nbuf = (uint32_t)min(kMaxNbuf, G::kAccCols / stride);
-  uint32_t it = 0;        // blocks so far, over all passes (expanders, MMA issuer, mask warps)
   uint32_t b = 0, ph = 0; // MMA issuer, mask warps: the next block's accumulator, and the parity of its use
   const auto first_acc = [&](uint32_t block) {
     b = block % nbuf;
@@ -381,11 +395,10 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
       ph ^= 1u;
     }
   };
-  uint32_t st_base = 0;   // ring stages so far (loader, expanders)
-  uint32_t issued = 0;    // loader: copies issued, stages 0 .. issued - 1
   uint32_t ep = 0;        // epilogue: reopenings so far (the epoch of the queue's ready stamps)
 
   for (int q0 = 0; q0 < a.B; q0 += kQC) {
+    const uint32_t it = (uint32_t)(q0 / kQC) * nb, st_base = (uint32_t)(q0 / kQC) * nstages;   // blocks, stages so far
     const int qn = min(kQC, a.B - q0);
     const int npad = (qn + 31) / 32 * 32;
     // ---- pass set-up (epilogue warps): the resident query operand, the lists and counters ----
@@ -426,43 +439,45 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
             break;
           }
           // the stage's entries, at most j_end: whole signatures of 16 W / 4 bytes, so a multiple of 16
-          const int64_t e0 = j_begin + (int64_t)si * G::kBPS * kBlockRows;
-          const uint32_t bytes = (uint32_t)min((int64_t)G::kBPS * kBlockRows, j_end - e0) * W * 4;
+          const uint32_t e0 = j_begin + si * G::kBPS * kBlockRows;
+          const uint32_t bytes = min((uint32_t)G::kBPS * kBlockRows, j_end - e0) * W * 4;
           mbar_expect_tx(full_bar(st), bytes);
           asm volatile(
               "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-              ::"r"(ring_smem + (uint32_t)st * kStageBytes), "l"(l.sig + e0 * W), "r"(bytes), "r"(full_bar(st))
+              ::"r"(ring_smem + (uint32_t)st * kStageBytes), "l"(l.sig + (int64_t)e0 * W), "r"(bytes), "r"(full_bar(st))
               : "memory");
-          issued = k + 1;
+          t.issued = k + 1;
         }
       }
       __syncwarp();
-      st_base += nstages;
     } else if (warp >= kEpiWarps && warp < kMmaWarp) {
       // ---------------- expanders ----------------
-      const int quad = warp % 4;
+      const int quad = warp % 4, set = (warp - kEpiWarps) / 4;
       const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
       bool ok = true;
-      // every block slot of the pass's stages, also those past the last block: each stage gets all its releases
-      for (uint32_t ti = 0; ti < nstages * G::kBPS; ++ti) {
+      // every kExpSets-th block slot of the pass's stages, also those past the last block: each stage gets all its
+      // releases
+      for (uint32_t ti = set; ti < nstages * G::kBPS; ti += kExpSets) {
         const uint32_t k = st_base + ti / G::kBPS;
         const int st = k % kS;
-        ok = __all_sync(kFull, mbar_wait_inline(full_bar(st), (k / kS) & 1u, abort_flag));
-        if (!ok) break;
-        const unsigned char* src = ring + (size_t)st * kStageBytes +
-                                   ((size_t)(ti % G::kBPS) * kBlockRows + quad * 32 + lane) * W * 4;
+        bool there = mbar_wait_inline(full_bar(st), (k / kS) & 1u, abort_flag);
         if (ti < nb) {
+          const unsigned char* src = ring + (size_t)st * kStageBytes +
+                                     ((size_t)(ti % G::kBPS) * kBlockRows + quad * 32 + lane) * W * 4;
+          uint4 y[W / 4];
+#pragma unroll
+          for (int h = 0; h < W / 4; ++h) y[h] = *reinterpret_cast<const uint4*>(src + 16 * h);
           const uint32_t u = it + ti;
-          const int b = u % kABuf;
-          ok = __all_sync(kFull, mbar_wait_inline(aempty_bar(b), ((u / kABuf) & 1u) ^ 1u, abort_flag));
+          const int b = u % G::kABuf;
+          there = there && mbar_wait_inline(aempty_bar(b), ((u / G::kABuf) & 1u) ^ 1u, abort_flag);
+          ok = __all_sync(kFull, there);
           if (!ok) break;
           tc_fence_after();
           const uint32_t dst = a_tmem + lane_addr + (uint32_t)(b * G::kACols);
-          // four signature words, 32 columns, at a time; rolled: the roles' loops share the instruction cache
-#pragma unroll 1
+          // four signature words, 32 columns, at a time
+#pragma unroll
           for (int h = 0; h < W / 4; ++h) {
-            const uint4 y = *reinterpret_cast<const uint4*>(src + 16 * h);
-            const uint32_t x[4] = {y.x, y.y, y.z, y.w};
+            const uint32_t x[4] = {y[h].x, y[h].y, y[h].z, y[h].w};
             uint32_t r[32];
 #pragma unroll
             for (int w = 0; w < 4; ++w)
@@ -474,18 +489,17 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
           tc_fence_before();
           __syncwarp();
           if (lane == 0) {
-            mbar_arrive(empty_bar(st));
             mbar_arrive(afull_bar(b));
+            mbar_arrive(empty_bar(st));
           }
         } else {   // past the last block: only the stage's release
-          __syncwarp();
+          ok = __all_sync(kFull, there);
+          if (!ok) break;
           if (lane == 0) mbar_arrive(empty_bar(st));
         }
       }
       if (!ok && lane == 0) fail();
       __syncwarp();
-      st_base += nstages;
-      it += nb;
     } else if (warp == kMmaWarp) {
       // ---------------- MMA issue ----------------
       // kind::f8f6f4: D f32 (bits 4-5 = 1), A and B e4m3 (bits 7-9, 10-12 = 0), both K-major, N >> 3 in bits 17-22,
@@ -494,9 +508,9 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
       const uint64_t qdesc = smem_desc(q_smem);
       first_acc(it);
       for (uint32_t ti = 0; ti < nb; ++ti) {
-        const uint32_t u = it + ti, ab = u % kABuf;
+        const uint32_t u = it + ti, ab = u % G::kABuf;
         if (!__all_sync(kFull, mbar_wait_inline(tempty_bar(b), ph ^ 1u, abort_flag) &&
-                                   mbar_wait_inline(afull_bar(ab), (u / kABuf) & 1u, abort_flag))) {
+                                   mbar_wait_inline(afull_bar(ab), (u / G::kABuf) & 1u, abort_flag))) {
           if (lane == 0) fail();
           break;
         }
@@ -516,7 +530,6 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
         __syncwarp();
         next_acc();
       }
-      it += nb;
     } else if (warp < kMaskWarps) {
       // ---------------- mask warps ----------------
       const int mw = warp;                                 // mask warp
@@ -533,22 +546,21 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
       first_acc(it);
       bool stop = false;
       for (uint32_t t0 = 0; t0 < nb && !stop; t0 += kRound) {
-        // Admitted pairs are rare: a first look at a block takes only the maximum of
-        // each 32-query chunk's scores; the admitted queries are told apart, and queued for the checker warps, where some
-        // lane's maximum reaches the threshold.
+        // Admitted pairs are rare: a first look at a block takes only the maximum of the chunk's scores; the admitted
+        // queries are told apart, and queued for the checker warps, where some lane's maximum reaches the threshold.
         bool got = true;
         int top = -1;            // the highest queue slot this thread took
-        uint32_t over = 0;       // bit r * kOwn + i: pairs of the warp's chunk i of block t0 + r found the queue full ...
-        uint32_t rest[kRound * kOwn];   // ... these (touched in that case only)
-        // queue the queries of `mask` (of chunk c) with entry j, as many as fit; the others are returned
-        auto push = [&](uint32_t mask, int c, int64_t j) -> uint32_t {
+        uint32_t over = 0;       // bit r: pairs of block t0 + r found the queue full ...
+        uint32_t rest[kRound];   // ... these (touched in that case only)
+        // queue the queries of `mask` with entry j, as many as fit; the others are returned
+        auto push = [&](uint32_t mask, uint32_t j) -> uint32_t {
           uint32_t full = 0;
           while (mask) {
             const int bit = __ffs(mask) - 1;
             mask &= mask - 1;
             const int slot = atomicAdd(&t.count, 1);
             if (slot < kCap) {
-              *reinterpret_cast<volatile uint64_t*>(&t.items[slot]) = pack_item(ep, 32 * c + bit, (int32_t)j);
+              *reinterpret_cast<volatile uint64_t*>(&t.items[slot]) = pack_item(ep, 32 * part + bit, (int32_t)j);
               top = slot;
             } else {
               full |= 1u << bit;
@@ -557,38 +569,44 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
           return full;
         };
         const auto entry = [&](int r) {   // this thread's entry of block t0 + r
-          return j_begin + (int64_t)(t0 + r) * kBlockRows + quad * 32 + lane;
+          return j_begin + (t0 + r) * kBlockRows + quad * 32 + lane;
         };
 #pragma unroll 1
-        for (int r = 0; r < kRound && t0 + r < nb; ++r) {
+        for (int r = 0; part < first_chunks && r < kRound && t0 + r < nb; ++r) {
           got = __all_sync(kFull, mbar_wait_inline(tfull_bar(b), ph, abort_flag));
           if (!got) break;   // the warp-collective loads below need the whole warp
           tc_fence_after();
           const uint32_t acc = tmem + lane_addr + b * (uint32_t)stride;
-#pragma unroll 1
-          for (int c = part; c < nch; c += kMaskParts) {
-            uint32_t v[32];
-            tmem_ld32_issue(acc + 32u * c, v);
-            tmem_ld32_wait(v);
-            if (!__any_sync(kFull, max32(v) >= thr)) continue;
-            uint32_t mask = 0;
-#pragma unroll
-            for (int i = 0; i < 32; ++i) mask |= (__uint_as_float(v[i]) >= thr ? 1u : 0u) << i;
-            const int left = qn - 32 * c;   // padding queries past qn are never admitted
-            if (left < 32) mask &= (1u << left) - 1u;
-            const int64_t j = entry(r);
-            const uint32_t full = j < j_end ? push(mask, c, j) : 0u;
-            if (full) {
-              const int i = r * kOwn + c / kMaskParts;
-              over |= 1u << i;
-              rest[i] = full;
-            }
-            __syncwarp();   // the load above is warp-collective
+          // the accumulator is free once its scores are in registers: the MMA issuer does not wait for what follows
+          const uint32_t free_bar = tempty_bar(b);
+          next_acc();
+          if (part >= nch) {   // no chunk of this pass's queries
+            if (lane == 0) mbar_arrive(free_bar);
+            continue;
           }
+          uint32_t v[32];
+          tmem_ld32_issue(acc + 32u * part, v);
+          tmem_ld32_wait(v);
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(tempty_bar(b));
-          next_acc();
+          if (lane == 0) mbar_arrive(free_bar);
+          if (__any_sync(kFull, max32(v) >= thr)) {
+            // the differences' signs, taken by a subtraction and a shift each (integers: no rounding, and no -0)
+            uint32_t mask = 0;
+#pragma unroll
+            for (int i = 31; i >= 0; --i)
+              mask = __funnelshift_l(__float_as_uint(__uint_as_float(v[i]) - thr), mask, 1);
+            mask = ~mask;
+            const int left = qn - 32 * part;   // padding queries past qn are never admitted
+            if (left < 32) mask &= (1u << left) - 1u;
+            const uint32_t j = entry(r);
+            const uint32_t full = j < j_end ? push(mask, j) : 0u;
+            if (full) {
+              over |= 1u << r;
+              rest[r] = full;
+            }
+            __syncwarp();   // the next load is warp-collective
+          }
         }
         // close the queue while it is past kFlushAt or a pair found it full, then queue the pairs that did (every
         // turn either queues all of them or fills the queue, so this ends). All mask warps leave together.
@@ -606,14 +624,13 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
           top = -1;
           for (uint32_t o = over; o; o &= o - 1) {
             const int i = __ffs(o) - 1;
-            rest[i] = push(rest[i], part + kMaskParts * (i % kOwn), entry(i / kOwn));
+            rest[i] = push(rest[i], entry(i));
             if (!rest[i]) over &= ~(1u << i);
           }
         }
       }
       // the pass's last close, also after a timeout: the checkers leave only at a reopening
       close(true);
-      it += nb;
     }
 
     if (warp < kEpiWarps) {
@@ -673,6 +690,7 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
   // nothing in flight when the CTA exits: the loader waits for its last kS copies (a consumed one passes at
   // once), the MMA issuer for every MMA; then TMEM is freed
   if (warp == kLoadWarp && lane == 0) {
+    const uint32_t issued = t.issued;
     for (uint32_t k = issued >= (uint32_t)kS ? issued - kS : 0u; k < issued; ++k)
       mbar_wait_inline(full_bar(k % kS), (k / kS) & 1u, nullptr);
   }

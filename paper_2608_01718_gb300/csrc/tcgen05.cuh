@@ -36,11 +36,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 }
 // Slow path of mbar_wait: poll until the phase completes, about a second passes, or another role aborts.
 __device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, const volatile uint32_t* abort_flag) {
-  const long long t0 = clock64();
+  long long t0 = 0;   // the clock is read only once the first probe has failed
   while (true) {
     if (mbar_try_wait(bar, parity)) return true;
     if (abort_flag && *abort_flag) return false;
-    if (clock64() - t0 > kWaitCycles) return false;
+    const long long now = clock64();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > kWaitCycles) return false;
   }
 }
 __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, const volatile uint32_t* abort_flag) {

@@ -170,7 +170,7 @@ def test_full_radius_equals_the_exact_scan_and_appends_are_signed(batch, bits):
 
 
 @pytest.mark.parametrize("n", [1, 127, 129, 255, 2_200, 38_913])
-@pytest.mark.parametrize("bits,batch", [(128, 129), (256, 48), (256, 300), (512, 97)])
+@pytest.mark.parametrize("bits,batch", [(128, 65), (128, 129), (256, 48), (256, 300), (512, 97)])
 def test_tensor_scan_block_and_pass_edges_equal_the_exact_scan(bits, batch, n):
     # the tensor-core scan at the edges of its 128-entry blocks and 8 KB stages (a ragged last block, one block per
     # split, 38,913 entries = 2 blocks on all splits and 3 on some), of its 128-query passes and of its 32-query
