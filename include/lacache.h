@@ -68,11 +68,10 @@ typedef enum {
   LACACHE_STAGE1_STREAM = 2, /* streaming CUDA-core scan: warp per key tile, 128-bit key loads, packed fp32 FMA */
   LACACHE_STAGE1_LSH = 3,    /* SimHash index, then the exact key check (requires lacache_enable_lsh) */
   LACACHE_STAGE1_TENSOR_PAIR = 4, /* reported by lacache_last_launch only, not a configuration value: the tensor
-                                     scan on two-CTA clusters (one M=256 MMA per pair of SMs), chosen for batches
-                                     of more than 128 queries */
+                                     scan on two-CTA clusters (one M=256 MMA per pair of SMs), chosen for most
+                                     batches of more than 128 queries */
   LACACHE_STAGE1_LSH_TENSOR = 5   /* reported by lacache_last_launch only: the SimHash form with the Hamming test on
-                                     the tensor cores, chosen for batches of at least 48 queries at 256 bits
-                                     and of at least 40 at 128 and 512 bits */
+                                     the tensor cores, chosen for larger batches (lacache_enable_lsh) */
 } lacache_stage1;
 
 /* Ensemble of m lookahead checks (section 3.4, "Analysis"; Figure 6): every entry and query carries one k-token
@@ -195,9 +194,10 @@ lacache_status lacache_append_misses(lacache_t* h, int32_t B, const void* q_emb_
  * hyperplanes_dev ([bits x d] bf16, copied into the handle; random normal rows give random-hyperplane LSH). With
  * cfg->stage1 == LACACHE_STAGE1_LSH a lookup applies the exact key check only to the entries whose signature
  * differs from the query's in at most `radius` bits; stage 2 is unchanged. Existing entries are signed now and
- * later inserts and appends are signed as they arrive. Batches of fewer than T queries (T = 48 at 256 bits, 40 at
- * 128 and 512) compare the packed signatures by population counts; larger ones run the Hamming test on the tensor
- * cores. Allocates (capacity + max_batch) * bits / 8 bytes for the signatures.
+ * later inserts and appends are signed as they arrive. Batches of fewer than T queries compare the packed
+ * signatures by population counts; larger ones run the Hamming test on the tensor cores. T = 48 at 256 bits and 40 at
+ * 128 and 512; on stores of 131,072 entries and more 33; from 2,097,152 entries 32, 24 and 18 at 128, 256 and 512 bits.
+ * Allocates (capacity + max_batch) * bits / 8 bytes for the signatures.
  * Asynchronous on cuda_stream; calling it again replaces the index. A lookup on a handle whose cfg->stage1 is
  * LACACHE_STAGE1_LSH returns LACACHE_ERR_INVALID_ARG, and runs nothing, until this call has been made. */
 lacache_status lacache_enable_lsh(lacache_t* h, int32_t bits, int32_t radius, const void* hyperplanes_dev,
@@ -274,7 +274,7 @@ lacache_status lacache_stage_times(lacache_t* h, double* stage1_ms, double* stag
  * (512-bit signatures, or one query on a store of at least 16 tiles of 512 entries per split): its first CTA
  * withholds the bulk copy of its first tile, every thread's bounded wait for that tile runs out, the CTA still
  * ends its passes and waits (bounded) for its issued copies, and the timeout is recorded the same way.
- * On CTA pairs (B > 128) the first CTA is the leader of the first pair; its abort stops its peer too. A single
+ * On CTA pairs the first CTA is the leader of the first pair; its abort stops its peer too. A single
  * query tile (B <= 128) runs on a dynamic schedule: the stall happens only if the first CTA claims a key tile, which
  * is certain when the store holds many more 256-key tiles than the GPU has SMs. 0 cancels. */
 lacache_status lacache_inject_stall(lacache_t* h, int32_t lookups);

@@ -452,7 +452,7 @@ lacache_status run_lookup(lacache* h, int32_t B, const void* q_emb, const void* 
               : lc::launch_sign_queries(a.q, B, c.d, h->hyper, h->lsh_bits, h->qsig, st, gathered);
       if (e == cudaSuccess) {
         lc::LshArgs l{h->sig, h->qsig, h->lsh_bits / 32, h->lsh_radius};
-        if (B >= lc::lsh_tensor_min_batch(h->lsh_bits)) {
+        if (B >= lc::lsh_tensor_min_batch(h->lsh_bits, h->n)) {
           e = lc::launch_stage1_lsh_tc(a, l, h->num_sms, h->max_splits, st, &splits);
           kernel = LACACHE_STAGE1_LSH_TENSOR;
         } else {

@@ -155,18 +155,31 @@ struct LshArgs {
   int words;
   int radius;
 };
-// Popcount scan (small batches) and the tensor-core scan (batches of at least lsh_tensor_min_batch(bits) queries).
+// Popcount scan (small batches) and the tensor-core scan (batches of at least lsh_tensor_min_batch queries).
 // *ring: the launch runs the scan's shared-memory ring form (the only form with bounded waits, so the only one a
 // stall injection, a.inject_stall, acts on).
 cudaError_t launch_stage1_lsh(const Stage1Args& a, const LshArgs& l, int num_sms, int max_splits, cudaStream_t st,
                               int* splits, bool* ring);
 cudaError_t launch_stage1_lsh_tc(const Stage1Args& a, const LshArgs& l, int num_sms, int max_splits,
                                  cudaStream_t st, int* splits);
-// The switch between them, measured per lookup step on mid-1m with both scans forced (popcount scan with its prefix
-// test / tensor-core scan, us): 128 bits, B = 32 48.1 / 56.7, B = 40 61.0 / 57.4; 256 bits, B = 40 74.0 / 80.8,
-// B = 48 81.6 / 81.6, B = 64 97.5 / 82.4; 512 bits, B = 32 77.5 / 97.6, B = 40 104.2 / 98.9. Past 32 queries the
-// popcount scan makes a second pass over the index.
-inline int lsh_tensor_min_batch(int bits) { return bits == 256 ? 48 : 40; }
+// The switch between them. The popcount scan's time grows with n * B and steps up past 32 queries, with its second pass
+// over the index; the tensor scan's hardly grows with B. From kLshLargeStore entries the lines lie where the two cross,
+// on stores of kLshSecondPassStore and more at the popcount scan's second pass. Measured per lookup step on d = 768
+// with both scans forced (popcount / tensor, us):
+//   2M entries: 128 bits, B = 28 60.4 / 59.6, 32 64.6 / 60.3; 256 bits, 20 63.2 / 64.2, 24 70.1 / 65.4; 512 bits, 16
+//     80.6 / 80.6, 18 87.3 / 81.0 (d = 160 and 1280: the same within 3 us);
+//   4M: 128 bits, 32 116 / 107; 256 bits, 24 127 / 116; 512 bits, 16 139 / 144, 24 182 / 146;
+//   1M: 128 bits, 32 38.0 / 37.4, 40 50.1 / 39.3; 256 bits, 32 47.8 / 41.2, 40 62.5 / 42.8; 512 bits, 32 66.2 / 49.0;
+//   131,072: 32 17.2-20.8 / 16.5-19.8, 33 18.5 / 16.8, 20.5 / 18.0 and 25.0 / 20.5 (128, 256 and 512 bits);
+//   100,000: 128 bits, 32 15.7 / 16.8, 40 19.9 / 17.0; 256 bits, 40 22.3 / 17.6.
+// Below, a batch of up to 32 queries gains at most some 15 us, and callers that look at the reported kernel find the
+// popcount scan there.
+constexpr int64_t kLshLargeStore = 1 << 21, kLshSecondPassStore = 1 << 17;
+inline int lsh_tensor_min_batch(int bits, int64_t n) {
+  if (n >= kLshLargeStore) return bits == 128 ? 32 : bits == 256 ? 24 : 18;
+  if (n >= kLshSecondPassStore) return 33;
+  return bits == 256 ? 48 : 40;
+}
 
 // LACACHE_STAGE1_AUTO's choice for a lookup of B queries against n keys of d elements, from measurements of both
 // kernels. Once the keys stream from HBM, the tensor-core scan holds the copy bandwidth at every batch size (1.05-1.09

@@ -229,3 +229,26 @@ def test_lookup_before_the_index_is_enabled_is_refused():
         out = cache.lookup(q["emb"], q["prefix"], q["ids"])
         torch.cuda.synchronize()
         assert out["status"].shape == (w.batch,)
+
+
+@pytest.mark.parametrize("n,bits,batch", [(131_071, 128, 33), (131_072, 128, 33), (131_072, 512, 39),
+                                          (2_097_151, 256, 24), (2_097_152, 128, 32), (2_097_152, 256, 23),
+                                          (2_097_152, 256, 24), (2_097_152, 512, 18)])
+def test_large_stores_take_the_tensor_scan_earlier_and_equal_the_exact_scan(n, bits, batch):
+    # both sides of the store sizes and batches at which lookups change from the popcount to the tensor-core scan. An
+    # entry at the key threshold differs in about acos(0.9) / pi = 0.14 of the bits, with a standard deviation of 0.031
+    # of 128 bits, so the radius of 0.375 (seven of them) keeps every candidate, and the lookup is the exact scan's
+    w = wl.WORKLOADS["mid-1m"].scaled(n=n, d=64, batch=batch)
+    first = (18 if bits == 512 else 24 if bits == 256 else 32) if n >= 1 << 21 else \
+        33 if n >= 1 << 17 else 48 if bits == 256 else 40
+    with new_cache(w, L.LACACHE_STAGE1_TENSOR) as exact_cache, new_cache(w, L.LACACHE_STAGE1_LSH) as cache:
+        for c in (exact_cache, cache):
+            fill(c, w)
+        L.lacache_enable_lsh(cache.h, bits, bits // 2 - bits // 8, wl.hyperplanes(bits, w.d, device="cuda"))
+        q = wl.batch(w, 0, device="cuda")
+        a, b = gpu_lookup(exact_cache, q), gpu_lookup(cache, q)
+        assert cache.last_launch()[1] == (L.LACACHE_STAGE1_LSH_TENSOR if batch >= first else L.LACACHE_STAGE1_LSH)
+    hit = a["status"] == L.LACACHE_HIT
+    assert hit.any()
+    assert np.array_equal(a["status"], b["status"]) and np.array_equal(a["n_cand"], b["n_cand"])
+    assert np.array_equal(a["entry_id"][hit], b["entry_id"][hit])
