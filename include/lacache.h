@@ -161,7 +161,8 @@ lacache_status lacache_lookup(lacache_t* h, int32_t B, const void* q_emb_dev, co
 /* lacache_lookup for host-resident queries and results (any host memory: pageable or pinned, any alignment).
  * The inputs reach the handle's device staging in one of two ways. An array in pinned memory that the device can
  * map is read by the device directly, one gather kernel covering all such arrays. Any other array is copied by
- * DMA. The same kernels then run. Their results go straight into the handle's mapped pinned staging, or through
+ * DMA. The same kernels then run. (A small batch whose three arrays the device can map, 16-byte aligned rows and
+ * 4-byte aligned ids, is not staged where the streaming scan takes it: the kernels read the arrays in place.) Their results go straight into the handle's mapped pinned staging, or through
  * one device-to-host copy where the device cannot map it. The call synchronizes cuda_stream, copies the results
  * into *out_host (host pointers) and returns. */
 lacache_status lacache_lookup_host(lacache_t* h, int32_t B, const void* q_emb_host, const void* q_prefix_host,
@@ -172,7 +173,8 @@ lacache_status lacache_lookup_host(lacache_t* h, int32_t B, const void* q_emb_ho
  * must lie in pinned host memory that the handle's device can map (cudaHostAlloc or cudaMallocHost, or
  * cudaHostRegister with mapping; with unified addressing all pinned memory is mapped), and each output field must
  * be aligned to its element size; otherwise the call returns LACACHE_ERR_INVALID_ARG and runs nothing. One kernel
- * gathers the inputs into the handle's device staging, the lookup's kernels follow, and they write the results
+ * gathers the inputs into the handle's device staging (small batches of the streaming scan are read in place, as by
+ * lacache_lookup_host), the lookup's kernels follow, and they write the results
  * straight into the output arrays. The call returns once they are enqueued on cuda_stream. The output arrays hold
  * the results, and the input arrays may be reused, only after the stream has passed the call (an event recorded
  * after it, or cudaStreamSynchronize). Calls on one handle must all use one stream: the staging is the handle's. */

@@ -4,20 +4,22 @@
 //
 //   D[m][n] = sum_k Q[qt*128 + m][k] * K[t*256 + n][k]      (bf16 operands, fp32 accumulation in TMEM)
 //
+// (Key tiles are of 256 keys; of 64 or 128 on stores too small to give every SM one of them: see tile_keys.)
+//
 // Layout of the work. One query tile (B <= 128): a dynamic schedule, in which CTAs claim 256-key tiles from a
 // global counter (one split per CTA), which balances the tail. Several query tiles: units are (query tile of
 // 128, split of the key tiles), walked by a persistent grid with the query tile varying fastest, so the CTAs that
-// run at the same time stream the same key range and share it through L2; more than one query tile runs on CTA
-// pairs (below). Each CTA:
-//   warp 0      TMA producer: per k-step, one 128x64 query box and one 256x64 key box (128-byte swizzle) into a
-//               4-stage shared-memory ring (mbarrier full/empty pairs);
+// run at the same time stream the same key range and share it through L2; most such batches run on CTA pairs
+// (below; see use_pairs). Each CTA:
+//   warp 0      TMA producer: per k-step, one query box of up to 128x64 and one 256x64 key box (128-byte swizzle) into
+//               a 4-stage shared-memory ring (mbarrier full/empty pairs);
 //   warp 1      MMA issuer: allocates 512 TMEM columns (two 128x256 fp32 accumulators) and issues
 //               tcgen05.mma kind::f16 (M=128, N=256, K=16) from one thread; tcgen05.commit frees ring stages
 //               and hands a finished accumulator to the epilogue;
 //   warps 2..5  epilogue: thread = query row (TMEM lane); reads its 256 scores with tcgen05.ld, keeps a sorted
 //               top_c of (score, id) in registers with the threshold max(tau_c, current c-th best), and finally
 //               writes the unit's partial list. Double-buffered accumulators overlap it with the next tile's MMAs.
-// Batches of more than one query tile run as CTA pairs (a two-CTA cluster on the two SMs of a TPC): one
+// A CTA pair (a two-CTA cluster on the two SMs of a TPC): one
 // tcgen05.mma.cta_group::2 of M=256 (two query tiles, one per SM), N=256, K=16 per step. Each SM loads its own
 // 128x64 query box and HALF of the key box (128 keys); the pair's tensor cores exchange the key halves, and each
 // SM's TMEM receives its own 128 query rows x 256 keys. Per SM and k-step that is 32 KB of TMA writes and of MMA
