@@ -714,8 +714,10 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
     for (uint32_t k = issued >= (uint32_t)kS ? issued - kS : 0u; k < issued; ++k)
       mbar_wait_inline(full_bar(k % kS), (k / kS) & 1u, nullptr);
   }
-  if (warp == kMmaWarp && lane == 0) {
-    mma_commit<false>(drain_bar, 0);
+  if (warp == kMmaWarp) {
+    // from the lane that issued the MMAs: a commit covers its own thread's only, and after a timeout some may still run
+    if (elect_one()) mma_commit<false>(drain_bar, 0);
+    __syncwarp();
     mbar_wait_inline(drain_bar, 0, nullptr);
   }
   tc_fence_before();
