@@ -431,7 +431,7 @@ lacache_status run_lookup(lacache* h, int32_t B, const void* q_emb, const void* 
       a.inject_stall = 1;
       --h->inject_stall;
     }
-    // the SimHash scan takes the injection only in its ring form (the launcher reports which form ran)
+    // the SimHash popcount scan takes the injection only in its ring form (the launcher reports which form ran)
     if (h->inject_stall > 0 && kernel == LACACHE_STAGE1_LSH) a.inject_stall = 1;
     cudaError_t e;
     if (kernel == LACACHE_STAGE1_TENSOR) {
@@ -455,6 +455,7 @@ lacache_status run_lookup(lacache* h, int32_t B, const void* q_emb, const void* 
         if (B >= lc::lsh_tensor_min_batch(h->lsh_bits, h->n)) {
           e = lc::launch_stage1_lsh_tc(a, l, h->num_sms, h->max_splits, st, &splits);
           kernel = LACACHE_STAGE1_LSH_TENSOR;
+          if (a.inject_stall) --h->inject_stall;
         } else {
           bool ring = false;
           e = lc::launch_stage1_lsh(a, l, h->num_sms, h->max_splits, st, &splits, &ring);

@@ -85,8 +85,8 @@ struct Stage1Args {
   uint64_t* part_cand;
   PartMeta* part_meta;
   unsigned int* dev_status;
-  int inject_stall;           // test support: CTA 0 of the tensor kernel, or of the SimHash scan's ring form,
-                              // withholds one load (see lacache.h)
+  int inject_stall;           // test support: CTA 0 of the tensor kernel, of the SimHash tensor scan or of the
+                              // popcount scan's ring form withholds one load (see lacache.h)
   int* tile_ctr;              // tensor kernel, one query tile: dynamic tile schedule on these two counters
                               // [next tile, CTAs done], zero at launch and zero again when the grid ends
                               // (nullptr: static schedule)

@@ -400,6 +400,7 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
   // the range's entries (ids are int32: so is the store's size)
   const uint32_t j_begin = g_begin * kBlockRows, j_end = min((uint32_t)a.n, (g_begin + nb) * kBlockRows);
   const uint32_t nstages = (nb + G::kBPS - 1) / G::kBPS;    // ring stages per pass
+  const bool withhold = a.inject_stall && s == 0;           // test support: the first stage's copy is not issued
   const int C = a.top_c;
   const float thr = (float)(G::kBits - 2 * l.radius);   // admitted iff dot >= b - 2 radius
   const int stride = 32 * first_chunks;
@@ -458,6 +459,7 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
             fail();
             break;
           }
+          if (withhold && k == 0) continue;   // nothing arrives on this stage: the expanders' wait runs out
           // the stage's entries, at most j_end: whole signatures of 16 W / 4 bytes, so a multiple of 16
           const uint32_t e0 = j_begin + si * G::kBPS * kBlockRows;
           const uint32_t bytes = min((uint32_t)G::kBPS * kBlockRows, j_end - e0) * W * 4;
@@ -711,7 +713,7 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
   // once), the MMA issuer for every MMA; then TMEM is freed
   if (warp == kLoadWarp && lane == 0) {
     const uint32_t issued = t.issued;
-    for (uint32_t k = issued >= (uint32_t)kS ? issued - kS : 0u; k < issued; ++k)
+    for (uint32_t k = max(issued >= (uint32_t)kS ? issued - kS : 0u, withhold ? 1u : 0u); k < issued; ++k)
       mbar_wait_inline(full_bar(k % kS), (k / kS) & 1u, nullptr);
   }
   if (warp == kMmaWarp) {

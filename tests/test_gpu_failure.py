@@ -9,7 +9,9 @@ freeing the pair's TMEM.
 
 The SimHash popcount scan's ring form (always taken at 512 bits) has the same test: its first CTA withholds the
 bulk copy of its first tile, every thread's bounded wait for it runs out, and the CTA ends its pass, waits (bounded)
-for the copies it did issue, and exits.
+for the copies it did issue, and exits. So has the SimHash tensor scan: its first CTA withholds the copy of its first
+signatures, its expanders' wait runs out, the loader, MMA, mask and checker warps stop, and the copies and MMAs in
+flight are waited for before TMEM is freed.
 """
 import pytest
 import torch
@@ -80,3 +82,34 @@ def test_simhash_ring_wait_timeout_is_reported_and_the_context_stays_usable():
         # the injection was taken by that lookup: the next one runs clean
         cache.lookup(q["emb"], q["prefix"], q["ids"])
         cache.sync()
+
+
+# 40,000 entries: two or three blocks a CTA, all loaded before the wait runs out, in one pass of queries and in three;
+# 200,000 at 512 bits: more stages than the ring holds, so the loader waits too, and a batch of 33, which the popcount
+# scan's ring form would take on a smaller store; a wide radius: pairs are queued and checked in the other CTAs meanwhile
+@pytest.mark.parametrize("n,bits,batch,radius", [(40_000, 128, 64, None), (40_000, 256, 300, None),
+                                                 (200_000, 512, 33, None), (200_000, 256, 128, 256)])
+def test_simhash_tensor_scan_wait_timeout_is_reported_and_the_context_stays_usable(n, bits, batch, radius):
+    w = wl.WORKLOADS["mid-1m"].scaled(n=n, d=64, batch=batch)
+    with L.LaCache(w.d, w.k, w.n, w.tau_c, w.tau_a, w.top_c, max_batch=w.batch,
+                   stage1=L.LACACHE_STAGE1_LSH) as cache:
+        for ch in wl.iter_store(w, "cuda"):
+            cache.insert(ch["key"], ch["prefix"], ch["ids"])
+        if radius is None:
+            radius = wl.lsh_radius(w.tau_c, bits)
+        L.lacache_enable_lsh(cache.h, bits, radius, wl.hyperplanes(bits, w.d, device="cuda"))
+        q = wl.batch(w, 0, device="cuda")
+        before = {k: v.clone() for k, v in cache.lookup(q["emb"], q["prefix"], q["ids"]).items()}
+        cache.sync()
+        L.lacache_inject_stall(cache.h, 1)
+        cache.lookup(q["emb"], q["prefix"], q["ids"])
+        assert cache.last_launch()[1] == L.LACACHE_STAGE1_LSH_TENSOR
+        with pytest.raises(L.LacacheError) as e:
+            cache.sync()
+        assert e.value.status == L.LACACHE_ERR_DEVICE_TIMEOUT
+        cache.sync()                                   # the status word was cleared
+        for _ in range(2):                             # the injection was taken: later lookups run clean
+            after = cache.lookup(q["emb"], q["prefix"], q["ids"])
+            cache.sync()
+            for k in ("status", "entry_id", "cand_id", "n_cand"):
+                assert torch.equal(after[k], before[k]), k
