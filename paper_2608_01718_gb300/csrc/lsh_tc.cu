@@ -120,6 +120,7 @@ struct Tail {
   uint32_t abort_flag;
   uint32_t tmem_slot;
   uint32_t issued;             // the loader's copies: stages 0 .. issued - 1
+  long long progress;          // clock64() of the last reopening: restarts the budget of the waits behind the mask warps
   uint64_t bars[2 * kS + 2 * kMaxABuf + 2 * kMaxNbuf + 1];   // ring full / empty, A full / empty, accumulator full /
                                                              // empty, drain
 };
@@ -327,6 +328,7 @@ __device__ __forceinline__ bool reopen(Tail& t, int ew, int lane) {
     t.count = 0;
     t.claim = 0;
     t.closed = 0;
+    *reinterpret_cast<volatile long long*>(&t.progress) = clock64();
   }
   epi_sync();
   return end;
@@ -374,6 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
     mbar_init(drain_bar, 1);
     t.abort_flag = 0;
     t.issued = 0;
+    t.progress = clock64();
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   for (int i = threadIdx.x; i < kCap; i += kThreads) t.items[i] = ~(uint64_t)0;   // no epoch
@@ -393,6 +396,11 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
     *abort_flag = 1u;
     atomicOr(a.dev_status, kDevTimeout);
   };
+  // The loader's, expanders' and MMA issuer's waits. All three stand still while the mask warps have the pairs of a round
+  // checked that found the queue full. A round may leave 524,288 of them, and at d = 8192 with lists of 32 the checks of
+  // so many take 0.8 s, most of one wait's budget. So it restarts at every reopening, of which those pairs allow a limited
+  // number: every reopening either takes all of them or fills the queue.
+  auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait_inline(bar, parity, abort_flag, &t.progress); };
 
   const int s = blockIdx.x;
   const int64_t nblocks = (a.n + kBlockRows - 1) / kBlockRows;
@@ -455,7 +463,7 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
         for (uint32_t si = 0; si < nstages; ++si) {
           const uint32_t k = st_base + si;
           const int st = k % kS;
-          if (!mbar_wait_inline(empty_bar(st), ((k / kS) & 1u) ^ 1u, abort_flag)) {
+          if (!wait(empty_bar(st), ((k / kS) & 1u) ^ 1u)) {
             fail();
             break;
           }
@@ -482,7 +490,7 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
       for (uint32_t ti = set; ti < nstages * G::kBPS; ti += kExpSets) {
         const uint32_t k = st_base + ti / G::kBPS;
         const int st = k % kS;
-        bool there = mbar_wait_inline(full_bar(st), (k / kS) & 1u, abort_flag);
+        bool there = wait(full_bar(st), (k / kS) & 1u);
         if (ti < nb) {
           const unsigned char* src = ring + (size_t)st * kStageBytes +
                                      ((size_t)(ti % G::kBPS) * kBlockRows + quad * 32 + lane) * W * 4;
@@ -491,7 +499,7 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
           for (int h = 0; h < W / 4; ++h) y[h] = *reinterpret_cast<const uint4*>(src + 16 * h);
           const uint32_t u = it + ti;
           const int b = u % G::kABuf;
-          there = there && mbar_wait_inline(aempty_bar(b), ((u / G::kABuf) & 1u) ^ 1u, abort_flag);
+          there = there && wait(aempty_bar(b), ((u / G::kABuf) & 1u) ^ 1u);
           ok = __all_sync(kFull, there);
           if (!ok) break;
           tc_fence_after();
@@ -531,8 +539,7 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
       first_acc(it);
       for (uint32_t ti = 0; ti < nb; ++ti) {
         const uint32_t u = it + ti, ab = u % G::kABuf;
-        if (!__all_sync(kFull, mbar_wait_inline(tempty_bar(b), ph ^ 1u, abort_flag) &&
-                                   mbar_wait_inline(afull_bar(ab), (u / G::kABuf) & 1u, abort_flag))) {
+        if (!__all_sync(kFull, wait(tempty_bar(b), ph ^ 1u) && wait(afull_bar(ab), (u / G::kABuf) & 1u))) {
           if (lane == 0) fail();
           break;
         }

@@ -34,15 +34,22 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Slow path of mbar_wait: poll until the phase completes, about a second passes, or another role aborts.
-__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, const volatile uint32_t* abort_flag) {
+// Slow path of mbar_wait: poll until the phase completes, about a second passes, or another role aborts. `progress`, if
+// given, is a clock64() value in shared memory that another role renews while it works on what the wait depends on: the
+// second then counts from the later of that and the wait's start.
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, const volatile uint32_t* abort_flag,
+                                          const volatile long long* progress = nullptr) {
   long long t0 = 0;   // the clock is read only once the first probe has failed
   while (true) {
     if (mbar_try_wait(bar, parity)) return true;
     if (abort_flag && *abort_flag) return false;
     const long long now = clock64();
     if (t0 == 0) t0 = now;
-    if (now - t0 > kWaitCycles) return false;
+    if (now - t0 > kWaitCycles) {
+      if (!progress) return false;
+      t0 = *progress;
+      if (now - t0 > kWaitCycles) return false;
+    }
   }
 }
 __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, const volatile uint32_t* abort_flag) {
@@ -57,8 +64,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const v
 }
 
 // As mbar_wait, all inline: for kernels short of registers, where a call would spill what lives across it.
-__device__ __forceinline__ bool mbar_wait_inline(uint32_t bar, uint32_t parity, const volatile uint32_t* abort_flag) {
-  return mbar_poll(bar, parity, abort_flag);
+__device__ __forceinline__ bool mbar_wait_inline(uint32_t bar, uint32_t parity, const volatile uint32_t* abort_flag,
+                                                 const volatile long long* progress = nullptr) {
+  return mbar_poll(bar, parity, abort_flag, progress);
 }
 
 // True in one lane of a converged warp. The operands of tcgen05.mma are warp-uniform registers: a loop that the whole

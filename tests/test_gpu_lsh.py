@@ -252,3 +252,36 @@ def test_large_stores_take_the_tensor_scan_earlier_and_equal_the_exact_scan(n, b
     assert hit.any()
     assert np.array_equal(a["status"], b["status"]) and np.array_equal(a["n_cand"], b["n_cand"])
     assert np.array_equal(a["entry_id"][hit], b["entry_id"][hit])
+
+
+@pytest.mark.slow
+def test_a_long_drain_of_the_queue_is_not_a_timeout():
+    # radius = bits on 48 blocks of 128 rows per CTA: a round of 32 blocks leaves 524,288 pairs to a queue of 4,096. Rows
+    # of 8,192 elements whose scores rise along each CTA's range, so that every pair enters a list of 32, make their
+    # checks take 0.8 s, and for that long the loader, the expanders and the MMA issuer stand still: nearly the budget of
+    # one wait, which has to count the drain's progress
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    per, d, batch, bits, top_c, chunk = 48 * 128, 8192, 128, 256, 32, 1 << 15
+    n = per * sms
+    g = torch.Generator(device="cuda").manual_seed(d)
+    u, v = torch.linalg.qr(torch.randn((d, 2), generator=g, device="cuda", dtype=torch.float64))[0].float().T
+    q = dict(emb=u.bfloat16().expand(batch, d).contiguous(),
+             prefix=torch.zeros((batch, 8), dtype=torch.bfloat16, device="cuda"),
+             ids=torch.zeros((batch, 1), dtype=torch.int32, device="cuda"))
+    with L.LaCache(d, 1, n, 0.3, 0.5, top_c, max_batch=batch, stage1=L.LACACHE_STAGE1_LSH, prefix_dims=[8],
+                   tau_a_models=[0.5]) as cache:
+        for r in range(0, n, chunk):
+            m = min(chunk, n - r)
+            a = (0.5 + 0.49 * ((r + torch.arange(m, device="cuda")) % per) / per).unsqueeze(1)
+            key = (a * u + (1 - a * a).sqrt() * v).bfloat16()
+            cache.insert(key, torch.zeros((m, 8), dtype=torch.bfloat16, device="cuda"),
+                         torch.zeros((m, 1), dtype=torch.int32, device="cuda"))
+        L.lacache_enable_lsh(cache.h, bits, bits, wl.hyperplanes(bits, d, device="cuda"))
+        got = gpu_lookup(cache, q)   # raises on a timeout
+        assert cache.last_launch()[1] == L.LACACHE_STAGE1_LSH_TENSOR
+    # the last row of every CTA's range is the same row, and the largest: a tie that goes to the lowest ids
+    want = per * np.arange(top_c, dtype=np.int32) + per - 1
+    assert np.all(got["cand_id"] == want) and np.all(got["cand_score"] == got["key_score"][:, None])
+    # an fp32 sum of 8,192 products of unit rows: within 8192 * 2^-24 * sum |x y| < 5e-4 of the exact one
+    best = float(key[-1].double() @ u.bfloat16().double())
+    assert np.allclose(got["key_score"], best, rtol=0, atol=5e-4)
