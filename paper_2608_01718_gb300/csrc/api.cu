@@ -642,6 +642,8 @@ lacache_status lacache_insert(lacache_t* h, int64_t n, const void* key_dev, cons
                                                     n * d, n * pd);
     e = cudaGetLastError();
   }
+  // A copy last: it orders the rows before the lookups behind it, which are programmatic dependents and may read the keys
+  // without a wait.
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->ids + h->n * k, ids_dev, (size_t)n * k * 4, cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess) e = sign_rows(h, h->n, n, st);

@@ -90,8 +90,8 @@ struct Stage1Args {
   int* tile_ctr;              // tensor kernel, one query tile: dynamic tile schedule on these two counters
                               // [next tile, CTAs done], zero at launch and zero again when the grid ends
                               // (nullptr: static schedule)
-  int inputs_from_previous;   // tensor kernel: the queries are written by the grid launched just before (the
-                              // host-input gather), so wait for it before reading anything
+  int inputs_from_previous;   // the queries are written by the grid launched just before (the host-input gather), so
+                              // wait for it before reading anything
   int q_host;                 // streaming kernel: q is mapped host memory
 };
 

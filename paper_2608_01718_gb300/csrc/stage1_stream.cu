@@ -216,15 +216,19 @@ __global__ void __launch_bounds__(kThreads, 1) stage1_stream_kernel(const Stream
   constexpr int64_t kStep = (int64_t)kWarps * KT;
   int64_t t0 = j_begin + (int64_t)warp * KT;
   // One query group and one load phase (a row of up to 1024 elements): each tile's loads are issued before the one
-  // before is reduced, and the first tile's before the queries are there.
+  // before is reduced, and the first tile's before the queries are there (after the wait below, where there is one).
   const bool ahead = groups == 1 && p.nph == 1;
-  if (ahead) load_phase(t0, j_end, 0);
+  if (ahead && !p.wait_first) load_phase(t0, j_end, 0);
 
   // Launched as a programmatic dependent of the previous grid on the stream (the previous lookup's stage 2, which
   // reads the partial lists this grid writes and writes nothing it reads): the scan runs alongside it, and every
   // thread waits for it only before writing the partial lists. When the queries come from the grid just before
-  // (the host-input gather), every thread waits here instead, before reading them.
-  if (p.wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // (the host-input gather), every thread waits here instead, before reading anything: the gather starts this grid
+  // early, so it orders nothing else that was written before it.
+  if (p.wait_first) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (ahead) load_phase(t0, j_end, 0);
+  }
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   for (int i = threadIdx.x; i < qpad * dc; i += kThreads) {

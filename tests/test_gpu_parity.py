@@ -647,3 +647,28 @@ def test_host_lookups_read_small_batches_in_place(d, batch):
         for o, g in zip(outs, want):
             for k, v in o.items():
                 assert np.array_equal(v.numpy(), g[k], equal_nan=True), k
+
+
+@pytest.mark.parametrize("batch", [2, 5], ids=["in-place", "gathered"])
+@pytest.mark.parametrize("stage1", PATHS)
+def test_host_lookups_right_after_an_fp32_insert_see_its_rows(stage1, batch):
+    # nothing is waited for between the inserts, whose conversion kernel writes the rows, and the host lookup, whose
+    # kernels are programmatic dependents (the streaming scan reads a batch of 2 in place and has one of 5 gathered)
+    w = wl.WORKLOADS["tiny-4k"].scaled(n=2_000, d=768, batch=batch, clusters=20)
+    st = oracle_store(w)
+    q = wl.batch(w, 0, device="cuda")
+    hq = {k: q[k].cpu().pin_memory() for k in ("emb", "prefix", "ids")}
+    rows = list(wl.iter_store(w, "cuda"))
+    oq, p = oracle_queries(q), params(w)
+    res = oracle.lookup(st, oq, p)
+    for _ in range(8):
+        with new_cache(w, stage1) as cache:
+            out = L.alloc_result(w.batch, w.top_c, "cpu", pinned=True)
+            stream = torch.cuda.current_stream()
+            for ch in rows:
+                cache.insert(ch["key"], ch["prefix"], ch["ids"], L.LACACHE_F32, cuda_stream=stream)
+            L.lacache_lookup_host_async(cache.h, hq["emb"], hq["prefix"], hq["ids"], out, stream)
+            stream.synchronize()
+            cache.sync()
+        rep = compare({k: v.numpy() for k, v in out.items()}, res, p, pair_scores=pair_scores_fn(st, oq))
+        assert rep.exact + rep.band == w.batch
