@@ -52,15 +52,15 @@ def test_signatures_match_the_oracle(bits):
 
 
 def _expected_lsh_kernel(batch, bits):
-    # the tensor-core scan from 48 queries at 256 bits and from 40 at 128 and 512 bits
+    # the tensor-core scan from 48 queries at 256 bits and from 40 at 128 and 512 bits (on stores of fewer than 131,072
+    # entries; the callers' larger ones see at most 32 queries, which the popcount scan has below 2,097,152 entries)
     return L.LACACHE_STAGE1_LSH_TENSOR if batch >= (48 if bits == 256 else 40) else L.LACACHE_STAGE1_LSH
 
 
 # popcount-1 / -2: a pass of fewer queries than one group of 8 (only their distances are computed);
 # tensor-40: the tensor-core scan at 128 and 512 bits, two passes of the popcount scan at 256 bits (its switch is at
 # 48);
-# popcount-36: two passes of 32 queries (the handle's max_batch is below the tensor scan's minimum, so it keeps no
-# expanded index); tensor-200: two passes of 128 queries at 128 and 256 bits, four of 64 at 512, ragged last pass
+# popcount-36: two passes of 32 queries; tensor-200: two passes of 128 queries, the last one ragged
 @pytest.mark.parametrize("batch", [1, 2, 5, 32, 36, 40, 64, 200],
                          ids=["popcount-1", "popcount-2", "popcount-5", "popcount-32", "popcount-36", "tensor-40",
                               "tensor-64", "tensor-200"])
@@ -139,8 +139,7 @@ def _check_lsh_lookup(w, bits, one_at_a_time=False):
 @pytest.mark.parametrize("batch", [16, 64], ids=["popcount", "tensor"])
 def test_full_radius_equals_the_exact_scan_and_appends_are_signed(batch, bits):
     # radius = bits admits every pair: the queue overflows on every tile (at 512 bits the popcount scan's ring form,
-    # whose queue is a quarter of the register form's), and appended entries must be signed (in both the packed
-    # and the expanded form) before the next lookup
+    # whose queue is a quarter of the register form's), and appended entries must be signed before the next lookup
     w = wl.WORKLOADS["serve-2m"].scaled(n=30_000, batch=batch, clusters=300)
     R = wl.hyperplanes(bits, w.d, device="cuda")
     with new_cache(w, L.LACACHE_STAGE1_TENSOR, capacity=w.n + 4 * w.batch) as exact_cache, \

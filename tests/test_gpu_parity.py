@@ -32,7 +32,8 @@ def library():
 
 
 def expected_kernel(stage1, batch):
-    """The tensor path runs batches of more than one query tile on CTA pairs."""
+    """The tensor path runs batches of more than one query tile on CTA pairs. (Not those of 3 or 5 tiles on larger stores
+    with rows on 256-byte boundaries, which no caller here uses: test_query_tile_edges_and_odd_tile_counts does.)"""
     return L.LACACHE_STAGE1_TENSOR_PAIR if stage1 == L.LACACHE_STAGE1_TENSOR and batch > 128 else stage1
 
 
@@ -672,3 +673,57 @@ def test_host_lookups_right_after_an_fp32_insert_see_its_rows(stage1, batch):
             cache.sync()
         rep = compare({k: v.numpy() for k, v in out.items()}, res, p, pair_scores=pair_scores_fn(st, oq))
         assert rep.exact + rep.band == w.batch
+
+
+@pytest.mark.parametrize("top_c,ensemble,k", [(1, False, 16), (4, True, 33), (8, True, 16), (16, False, 37),
+                                              (16, True, 16), (32, False, 5), (32, True, 40)])
+def test_in_place_host_lookups_for_every_list_size_and_ensembles(top_c, ensemble, k):
+    # the second stage that stages its query in shared memory, for every list size (4, 8, 16 and 32 slots), one check and
+    # an ensemble of three (prefix rows of 2,176 elements), token ids past one warp's first 32. A batch of 3 at d = 768 is
+    # read in place on the streaming scan; the device lookup of the same queries is the reference, bit for bit.
+    w = wl.WORKLOADS["ensemble-1m" if ensemble else "mid-1m"].scaled(n=9_000, batch=3, clusters=30, top_c=top_c, k=k)
+    with new_cache(w, L.LACACHE_STAGE1_STREAM) as cache:
+        fill(cache, w)
+        for step in range(3):
+            q = wl.batch(w, step, device="cuda")
+            g = gpu_lookup(cache, q)
+            assert (g["n_cand"] > 0).any()
+            hq = {key: q[key].cpu().pin_memory() for key in ("emb", "prefix", "ids")}
+            out = L.alloc_result(w.batch, w.top_c, "cpu", pinned=True, models=cache.models)
+            L.lacache_lookup_host(cache.h, hq["emb"], hq["prefix"], hq["ids"], out)
+            for key, v in out.items():
+                assert np.array_equal(v.numpy(), g[key], equal_nan=True), key
+
+
+@pytest.mark.parametrize("offsets", [(2, 0, 0), (0, 8, 0), (0, 0, 4), (14, 2, 12)],
+                         ids=["emb", "prefix", "ids-in-place", "all"])
+def test_small_host_batches_off_16_byte_boundaries(offsets):
+    # small batches of the streaming scan whose key or prefix rows start off 16-byte boundaries are gathered instead of
+    # read in place; token ids need 4 bytes only
+    w = wl.WORKLOADS["mid-1m"].scaled(n=9_000, batch=2, clusters=30)
+    with new_cache(w, L.LACACHE_STAGE1_STREAM) as cache:
+        fill(cache, w)
+        stream = torch.cuda.current_stream()
+        for step in range(3):
+            q = wl.batch(w, step, device="cuda")
+            g = gpu_lookup(cache, q)
+            hq = {key: _host_copy(q[key], "pinned", off) for key, off in zip(("emb", "prefix", "ids"), offsets)}
+            out = L.alloc_result(w.batch, w.top_c, "cpu", pinned=True)
+            out2 = L.alloc_result(w.batch, w.top_c, "cpu", pinned=True)
+            L.lacache_lookup_host(cache.h, hq["emb"], hq["prefix"], hq["ids"], out)
+            L.lacache_lookup_host_async(cache.h, hq["emb"], hq["prefix"], hq["ids"], out2, stream)
+            stream.synchronize()
+            cache.sync()
+            for o in (out, out2):
+                for key, v in o.items():
+                    assert np.array_equal(v.numpy(), g[key], equal_nan=True), key
+
+
+@pytest.mark.parametrize("top_c,ensemble", [(1, False), (4, False), (8, False), (32, False), (8, True), (32, True)])
+def test_second_stage_of_large_batches(top_c, ensemble):
+    # from 1,024 queries the second stage runs four warps per query: every list size (16 slots: the full-size batch), one
+    # check and an ensemble, with full lists (60 entries per cluster)
+    w = wl.WORKLOADS["ensemble-1m" if ensemble else "serve-2m"].scaled(n=9_000, batch=1_030, clusters=150, top_c=top_c)
+    rep = run_parity(w, L.LACACHE_STAGE1_TENSOR)
+    assert rep.exact + rep.band == w.batch and rep.band <= w.batch // 10
+    assert rep.hits > 0 and rep.rejects > 0 and rep.misses > 0
