@@ -66,8 +66,9 @@ __host__ __device__ __forceinline__ float cand_score(uint64_t c) { return score_
 __host__ __device__ __forceinline__ uint32_t cand_id(uint64_t c) { return ~(uint32_t)c; }
 
 // Stage-1 output, per split s and query q: a record of the split's best key score (over all its entries: a miss
-// reports the best over the store) and of how many candidates its partial list holds, and the list itself, sorted,
-// in its first `count` slots (later slots are not written: most lists hold few candidates, or none).
+// reports the best over the store) and of how many candidates its partial list holds, and the list itself in its first
+// `count` slots, in any order (the SimHash tensor scan's is not sorted); later slots are not written: most lists hold few
+// candidates, or none.
 //   part_meta[s * B + q], part_cand[(s * B + q) * top_c + i] for i < count
 struct __align__(8) PartMeta {
   float best;
@@ -164,16 +165,18 @@ cudaError_t launch_stage1_lsh_tc(const Stage1Args& a, const LshArgs& l, int num_
                                  cudaStream_t st, int* splits);
 // The switch between them. The popcount scan's time grows with n * B and steps up past 32 queries, with its second pass
 // over the index; the tensor scan's hardly grows with B. From kLshLargeStore entries the lines lie where the two cross,
-// on stores of kLshSecondPassStore and more at the popcount scan's second pass. Measured per lookup step on d = 768
-// with both scans forced (popcount / tensor, us):
+// from kLshSecondPassStore at the popcount scan's second pass, and below at 48 and 40 queries, where the popcount scan and
+// the earlier tensor scan over an expanded index crossed. Measured per lookup step on d = 768 with both scans forced
+// (popcount / tensor, us):
 //   2M entries: 128 bits, B = 28 60.4 / 59.6, 32 64.6 / 60.3; 256 bits, 20 63.2 / 64.2, 24 70.1 / 65.4; 512 bits, 16
 //     80.6 / 80.6, 18 87.3 / 81.0 (d = 160 and 1280: the same within 3 us);
 //   4M: 128 bits, 32 116 / 107; 256 bits, 24 127 / 116; 512 bits, 16 139 / 144, 24 182 / 146;
 //   1M: 128 bits, 32 38.0 / 37.4, 40 50.1 / 39.3; 256 bits, 32 47.8 / 41.2, 40 62.5 / 42.8; 512 bits, 32 66.2 / 49.0;
 //   131,072: 32 17.2-20.8 / 16.5-19.8, 33 18.5 / 16.8, 20.5 / 18.0 and 25.0 / 20.5 (128, 256 and 512 bits);
 //   100,000: 128 bits, 32 15.7 / 16.8, 40 19.9 / 17.0; 256 bits, 40 22.3 / 17.6.
-// Below, a batch of up to 32 queries gains at most some 15 us, and callers that look at the reported kernel find the
-// popcount scan there.
+// So the lines below kLshLargeStore are on the popcount scan's side of the crossing: at 32 queries on 1M entries it is
+// 7 us behind at 256 bits and 17 at 512, further just below 2M, where its time has doubled, and 5 us at 40 queries on
+// 100,000 entries at 256 bits. The GPU tests expect it there (32 queries on 1M entries are its full-size case).
 constexpr int64_t kLshLargeStore = 1 << 21, kLshSecondPassStore = 1 << 17;
 inline int lsh_tensor_min_batch(int bits, int64_t n) {
   if (n >= kLshLargeStore) return bits == 128 ? 32 : bits == 256 ? 24 : 18;
@@ -193,10 +196,11 @@ inline int lsh_tensor_min_batch(int bits, int64_t n) {
 // 13.3, B = 2: 13.6 against 13.1. A single lookup on an idle device crosses later (16,384 x 768, B = 4: 18.2
 // against 21.2 us), and from a flushed L2 the streaming scan's stage 1 is also the shorter one at that size (22.3
 // against 25.9 us at 43,690 x 768, B = 1). So the streaming scan takes the lookups with n d B <= 2^25 (at most
-// 64 MiB of keys, at one query). Since the tensor-core scan takes such stores in tiles of 64 or 128 keys, it is level with
-// the streaming scan at 4 to 16 queries (4,096 x 384, stream / tensor: B = 4 7.5 / 7.1, B = 16 8.5 / 7.1) and well ahead
-// beyond (1,000 x 384: B = 32 13.8 / 8.3, B = 64 23.4 / 8.4; 4,096 x 128: B = 64 15.3 / 7.2), so batches of more than 24
-// queries, three of the streaming scan's query groups, go to it whatever their size.
+// 64 MiB of keys, at one query). Since the tensor-core scan takes such stores in tiles of 64 or 128 keys, it is well
+// ahead past 24 queries, three of the streaming scan's query groups (1,000 x 384, stream / tensor: B = 32 13.8 / 8.3,
+// B = 64 23.4 / 8.4; 4,096 x 128: B = 64 15.3 / 7.2), so those batches go to it whatever their size. From 4 to 24 it is
+// ahead by less (4,096 x 384: B = 4 7.5 / 7.1, B = 16 8.5 / 7.1); those keep the n d B line, where the GPU tests expect the
+// streaming scan (21 queries on 4,096 x 384).
 constexpr int64_t kStreamAutoMacs = (int64_t)1 << 25;
 constexpr int kStreamAutoBatch = 24;
 inline int auto_stage1(int64_t n, int d, int B) {

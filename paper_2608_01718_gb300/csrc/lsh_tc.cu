@@ -92,7 +92,7 @@ struct TcGeo {
   static constexpr int kQueryBytes = kQC * kBits;              // 16, 32 or 64 KB
   static constexpr int kABuf = W == 4 ? 4 : 2;
   static constexpr int kACols = 8 * W;
-  static constexpr int kAccCols = 512 - kABuf * kACols;        // 448, 384 or 256
+  static constexpr int kAccCols = 512 - kABuf * kACols;        // 384, 384 or 256
 };
 constexpr int kChunks = kQC / 32;                        // 32-query chunks of a block (at most)
 static_assert(kMaskParts == kChunks, "a mask warp has one chunk");

@@ -13,7 +13,8 @@
 // (below; see use_pairs). Each CTA:
 //   warp 0      TMA producer: per k-step, one query box of up to 128x64 and one 256x64 key box (128-byte swizzle) into
 //               a 4-stage shared-memory ring (mbarrier full/empty pairs);
-//   warp 1      MMA issuer: allocates 512 TMEM columns (two 128x256 fp32 accumulators) and issues
+//   warp 1      MMA issuer: allocates 512 TMEM columns (two 128x256 fp32 accumulators; 128 or 256 columns for tiles of
+//               64 or 128 keys) and issues
 //               tcgen05.mma kind::f16 (M=128, N=256, K=16) from one thread; tcgen05.commit frees ring stages
 //               and hands a finished accumulator to the epilogue;
 //   warps 2..5  epilogue: thread = query row (TMEM lane); reads its 256 scores with tcgen05.ld, keeps a sorted

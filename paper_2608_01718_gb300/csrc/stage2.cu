@@ -4,7 +4,7 @@
 //  1. merge the stage-1 partial lists (per split a record of its best score and candidate count, and that many
 //     packed candidates) into C_q, the top_c candidates by (key score desc, entry id asc): every thread keeps a
 //     sorted top-c of the candidates it reads (four splits in flight), each warp reduces its lanes' lists by top_c
-//     rounds of a warp-wide max, and warp 0 merges the eight warp lists the same way;
+//     rounds of a warp-wide max, and warp 0 merges the warps' lists the same way;
 //  2. the candidates are checked in parallel, one warp per candidate: r = <p_q, P_j> (the prefix-embedding cosine
 //     sim(f_k(x), f_k(x'))) in fp32, each lane's 8-element chunks in order, then a butterfly sum (every lane ends
 //     with the same bits); m = number of positions i < k with equal token ids;
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kWarps * 32, (kWarps == 8 ? 1 : 2) * (CPAD <= 
     }
   }
   __syncthreads();
-  // 1d. warp 0 merges the eight warp lists: lane l < kWarps walks list l
+  // 1d. warp 0 merges the warps' lists: lane l < kWarps walks list l
   if (warp == 0) {
     int head = 0;
     int n = 0;

@@ -81,8 +81,8 @@ def test_large_cache_near_hbm_capacity():
 
 
 def test_large_cache_through_the_simhash_index():
-    """16,777,216 entries x 1024 looked up through a 256-bit SimHash index (B = 128: the tensor-core Hamming scan
-    over the expanded index), every query of the batch against the streamed oracle. Queries whose outcome an
+    """16,777,216 entries x 1024 looked up through a 256-bit SimHash index (B = 128: the tensor-core Hamming
+    scan), every query of the batch against the streamed oracle. Queries whose outcome an
     ambiguous signature bit could change are set aside (at most 1 in 50)."""
     w = wl.WORKLOADS["large-16m"]
     bits = 256
