@@ -162,9 +162,9 @@ lacache_status lacache_lookup(lacache_t* h, int32_t B, const void* q_emb_dev, co
  * The inputs reach the handle's device staging in one of two ways. An array in pinned memory that the device can
  * map is read by the device directly, one gather kernel covering all such arrays. Any other array is copied by
  * DMA. The same kernels then run. (A small batch whose three arrays the device can map, 16-byte aligned rows and
- * 4-byte aligned ids, is not staged where the streaming scan takes it: the kernels read the arrays in place.) Their results go straight into the handle's mapped pinned staging, or through
- * one device-to-host copy where the device cannot map it. The call synchronizes cuda_stream, copies the results
- * into *out_host (host pointers) and returns. */
+ * 4-byte aligned ids, is not staged where the streaming scan takes it: the kernels read the arrays in place.) Their
+ * results go straight into the handle's mapped pinned staging, or through one device-to-host copy where the device
+ * cannot map it. The call synchronizes cuda_stream, copies the results into *out_host (host pointers) and returns. */
 lacache_status lacache_lookup_host(lacache_t* h, int32_t B, const void* q_emb_host, const void* q_prefix_host,
                                    const int32_t* q_ids_host, const lacache_result* out_host, void* cuda_stream);
 

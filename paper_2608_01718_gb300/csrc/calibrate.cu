@@ -149,9 +149,9 @@ __global__ void __launch_bounds__(kBins / 2)
 // t + 2 T, ... (T threads in all, at most kPer each). Each pass counts into the CTA's own shared histogram; after a
 // cluster barrier every CTA adds up all G histograms (through distributed shared memory) and picks the same bin.
 // Bound by latency. A call (similarities included), against separate kernels for the set-up and for each pass's count
-// and pick (us, before / after): 500 pairs x 1024 37.4 / 10.0, 5,000 x 384 41.0 / 12.4, 16,384 x 768 45.2 / 30.8,
-// 60,000 x 384 55.4 / 43.2, 131,072 x 768 100.5 / 100.5. Past that the values no longer fit the cluster's registers, and
-// counting on all SMs is as fast.
+// and pick (us, calls back to back, before / after): 500 pairs x 1024 39.0 / 10.7, 5,000 x 384 41.0 / 12.3, 16,384 x 768
+// 45.1 / 24.7, 60,000 x 384 53.3 / 41.0, 131,072 x 768 98.4 / 95.5. Past that the values no longer fit the cluster's
+// registers, and counting on all SMs is as fast.
 constexpr int kSelThreads = 1024;
 constexpr int kPer = 16;
 constexpr int kSelCluster = 8;

@@ -198,9 +198,9 @@ inline int lsh_tensor_min_batch(int bits, int64_t n) {
 // against 25.9 us at 43,690 x 768, B = 1). So the streaming scan takes the lookups with n d B <= 2^25 (at most
 // 64 MiB of keys, at one query). Since the tensor-core scan takes such stores in tiles of 64 or 128 keys, it is well
 // ahead past 24 queries, three of the streaming scan's query groups (1,000 x 384, stream / tensor: B = 32 13.8 / 8.3,
-// B = 64 23.4 / 8.4; 4,096 x 128: B = 64 15.3 / 7.2), so those batches go to it whatever their size. From 4 to 24 it is
-// ahead by less (4,096 x 384: B = 4 7.5 / 7.1, B = 16 8.5 / 7.1); those keep the n d B line, where the GPU tests expect the
-// streaming scan (21 queries on 4,096 x 384).
+// B = 64 23.4 / 8.4; 4,096 x 128: B = 64 15.3 / 7.2), so those batches go to it whatever their size. Up to 8 the two are
+// level there, and from 16 it is ahead too (4,096 x 384: B = 4 6.1 / 6.5, B = 8 6.5 / 6.6, B = 16 8.3 / 6.7, B = 21 10.0 /
+// 6.7); those batches keep the n d B line, where the GPU tests expect the streaming scan (21 queries on 4,096 x 384).
 constexpr int64_t kStreamAutoMacs = (int64_t)1 << 25;
 constexpr int kStreamAutoBatch = 24;
 inline int auto_stage1(int64_t n, int d, int B) {

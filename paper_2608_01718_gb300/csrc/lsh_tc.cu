@@ -46,9 +46,9 @@
 // barrier only every 32 blocks (every 16: 2 % slower). Six checker warps: with four, 128 queries take 179 instead of
 // 171; two pairs a checker at a time, or more A buffers, give nothing.
 // Measured per lookup step (us) against the scan over an index kept expanded in HBM that was here first / against one
-// expander set and late release: 4M x 768, 256 bits, 48 queries 177 / 172 -> 126, 64 180 / 174 -> 129, 128 202 / 188 ->
-// 163, 384 563 / 536 -> 464; 128 bits, 48 queries 131 / 133 -> 115, 128 184 / 163 -> 146; 512 bits, 64 queries 326 / 232
-// -> 175, 128 631 / 253 -> 225. (Without the mask warps' help at the end of the range 128 queries on 4M x 1024 take 18 %
+// expander set and late release: 4M x 768, 256 bits, 48 queries 176 / 172 -> 127, 64 180 / 174 -> 130, 128 202 / 188 ->
+// 167, 384 563 / 536 -> 471; 128 bits, 48 queries 132 / 133 -> 116, 128 188 / 163 -> 149; 512 bits, 64 queries 326 / 232
+// -> 176, 128 631 / 253 -> 225. (Without the mask warps' help at the end of the range 128 queries on 4M x 1024 take 18 %
 // longer, and 357 on 36,433 x 768 a fifth.) The packed index takes an eighth of the expanded one's memory, and signing
 // entries no second kernel.
 #include "internal.cuh"
