@@ -25,9 +25,9 @@
 //   warps 16-21 (checker warps): claim queued pairs as they arrive, compute their exact fp32 key scores over the
 //     gathered key rows (each lane's 8-element chunks in order, then a butterfly sum) while the scan goes on, and
 //     fold each score into its query's best score and, if it clears tau_c, into the query's list (lock-free). The
-//     mask warps join them once the range is scanned.
-// When the queue passes three quarters of its capacity, and at the end of the range, the mask warps close it: the
-// checkers finish what was queued below the close, then the queue is emptied and reopened in a new epoch. A pair
+//     mask warps join them at every close of the queue.
+// When the queue passes three quarters of its capacity, and at the end of the range, the mask warps close it: all checking
+// warps finish what was queued below the close, then the queue is emptied and reopened in a new epoch. A pair
 // that finds the queue full stays with its thread and is queued after the reopening. All
 // epilogue warps expand the pass's query signatures into the query operand and write the lists out. The checker
 // warps leave their loop only at a reopening, which the mask warps always run at the end of a pass, also after a
@@ -46,11 +46,14 @@
 // barrier only every 32 blocks (every 16: 2 % slower). Six checker warps: with four, 128 queries take 179 instead of
 // 171; two pairs a checker at a time, or more A buffers, give nothing.
 // Measured per lookup step (us) against the scan over an index kept expanded in HBM that was here first / against one
-// expander set and late release: 4M x 768, 256 bits, 48 queries 176 / 172 -> 127, 64 180 / 174 -> 130, 128 202 / 188 ->
-// 167, 384 563 / 536 -> 471; 128 bits, 48 queries 132 / 133 -> 116, 128 188 / 163 -> 149; 512 bits, 64 queries 326 / 232
-// -> 176, 128 631 / 253 -> 225. (Without the mask warps' help at the end of the range 128 queries on 4M x 1024 take 18 %
-// longer, and 357 on 36,433 x 768 a fifth.) The packed index takes an eighth of the expanded one's memory, and signing
-// entries no second kernel.
+// expander set and late release: 4M x 768, 256 bits, 48 queries 176 / 172 -> 120, 64 180 / 174 -> 123, 128 202 / 188 ->
+// 160, 384 563 / 536 -> 452; 128 bits, 48 queries 132 / 133 -> 108, 128 188 / 163 -> 144; 512 bits, 64 queries 326 / 232
+// -> 174, 128 631 / 253 -> 225. The packed index takes an eighth of the expanded one's memory, and signing entries no
+// second kernel.
+// The mask warps' help counts where many pairs are admitted. At the end of the range: without it 128 queries on 4M x 1024
+// take 18 % longer, and 357 on 36,433 x 768 a fifth. At the closes before: 1M x 768 in 64 clusters, 256 bits at radius 60,
+// 48 queries 859 -> 310, 128 2,050 -> 784 (the scan over the expanded index 450 and 1,128); 4,096 clusters, radius 112, 64
+// queries 2,393 -> 859 (1,146).
 #include "internal.cuh"
 #include "tcgen05.cuh"
 
@@ -66,7 +69,7 @@ constexpr int kExpWarps = 4 * kExpSets;                  // warps 22-29: expand 
 constexpr int kMmaWarp = kEpiWarps + kExpWarps;          // warp 30
 constexpr int kLoadWarp = kMmaWarp + 1;                  // warp 31
 constexpr int kThreads = (kLoadWarp + 1) * 32;
-// Queue capacity. A close before the end of the range stalls the scan until the checkers are done, so the queue holds what
+// Queue capacity. A close before the end of the range stalls the scan until the checks are done, so the queue holds what
 // a CTA usually queues in a whole range: 600 pairs on 4M entries in clusters of a thousand, 2,400 on a Zipf-skewed store of
 // 16.8M x 1024, where a lookup of 128 queries takes 1.02 ms with 1,024, 0.90 with 2,048 and 0.71 with 4,096.
 constexpr int kCap = 4096;
@@ -398,8 +401,8 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
   };
   // The loader's, expanders' and MMA issuer's waits. All three stand still while the mask warps have the pairs of a round
   // checked that found the queue full. A round may leave 524,288 of them, and at d = 8192 with lists of 32 the checks of
-  // so many take 0.8 s, most of one wait's budget. So it restarts at every reopening, of which those pairs allow a limited
-  // number: every reopening either takes all of them or fills the queue.
+  // so many take 0.26 s (0.8 s by the checker warps alone), much of one wait's budget. So it restarts at every reopening, of
+  // which those pairs allow a limited number: every reopening either takes all of them or fills the queue.
   auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait_inline(bar, parity, abort_flag, &t.progress); };
 
   const int s = blockIdx.x;
@@ -559,53 +562,40 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
         __syncwarp();
         next_acc();
       }
-    } else if (warp < kMaskWarps) {
-      // ---------------- mask warps ----------------
-      const int mw = warp;                                 // mask warp
-      const int quad = mw % 4, part = mw / 4;              // TMEM lane quadrant; column chunk(s) part + kMaskParts i
-      const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
-      // close the queue (every mask warp has queued its pairs)
-      auto close = [&](bool last) {
-        if (mw == 0 && lane == 0) {
-          if (last) t.pass_end = 1;
-          st_volatile(&t.closed, 1u + (uint32_t)min(t.count, kCap));
+    }
+
+    if (warp < kEpiWarps) {
+      // ---------------- mask warps: scan; checker warps, and the mask warps at a close: check ----------------
+      const int quad = warp % 4, part = warp / 4;            // mask warps: TMEM lane quadrant; 32-query column chunk
+      const int nch = npad / 32;                             // 32-query chunks of a block
+      // A mask thread's pairs that found the queue full: the queries per block of a round; which blocks have some; the
+      // round's first block. (Local memory: touched only when the queue fills up.)
+      uint32_t rest[kRound + 2];
+      // queue the queries of `mask` with entry j, as many as fit; the others are returned
+      auto push = [&](uint32_t mask, uint32_t j) -> uint32_t {
+        uint32_t full = 0;
+        while (mask) {
+          const int bit = __ffs(mask) - 1;
+          mask &= mask - 1;
+          const int slot = atomicAdd(&t.count, 1);
+          if (slot < kCap)
+            *reinterpret_cast<volatile uint64_t*>(&t.items[slot]) = pack_item(ep, 32 * part + bit, (int32_t)j);
+          else
+            full |= 1u << bit;
         }
+        return full;
       };
-      const int nch = npad / 32;                           // 32-query chunks of a block
-      first_acc(it);
-      bool stop = false;
-      for (uint32_t t0 = 0; t0 < nb && !stop; t0 += kRound) {
-        // Admitted pairs are rare: a first look at a block takes only the maximum of the chunk's scores; the admitted
-        // queries are told apart, and queued for the checker warps, where some lane's maximum reaches the threshold.
-        bool got = true;
-        int top = -1;            // the highest queue slot this thread took
-        uint32_t over = 0;       // bit r: pairs of block t0 + r found the queue full ...
-        uint32_t rest[kRound];   // ... these (touched in that case only)
-        // queue the queries of `mask` with entry j, as many as fit; the others are returned
-        auto push = [&](uint32_t mask, uint32_t j) -> uint32_t {
-          uint32_t full = 0;
-          while (mask) {
-            const int bit = __ffs(mask) - 1;
-            mask &= mask - 1;
-            const int slot = atomicAdd(&t.count, 1);
-            if (slot < kCap) {
-              *reinterpret_cast<volatile uint64_t*>(&t.items[slot]) = pack_item(ep, 32 * part + bit, (int32_t)j);
-              top = slot;
-            } else {
-              full |= 1u << bit;
-            }
-          }
-          return full;
-        };
-        const auto entry = [&](int r) {   // this thread's entry of block t0 + r
-          return j_begin + (t0 + r) * kBlockRows + quad * 32 + lane;
-        };
+      const auto entry = [&](uint32_t block) { return j_begin + block * kBlockRows + quad * 32 + lane; };   // this thread's
+      // A round: the blocks from t0 on, at most kRound. False after a timeout. Admitted pairs are rare: a first look at a block
+      // takes only the maximum of the chunk's scores; the admitted queries are told apart, and queued for the checker
+      // warps, where some lane's maximum reaches the threshold.
+      auto scan_round = [&](uint32_t t0) -> bool {
 #pragma unroll 1
         for (int r = 0; part < first_chunks && r < kRound && t0 + r < nb; ++r) {
-          got = __all_sync(kFull, mbar_wait_inline(tfull_bar(b), ph, abort_flag));
-          if (!got) break;   // the warp-collective loads below need the whole warp
+          // the warp-collective loads below need the whole warp
+          if (!__all_sync(kFull, mbar_wait_inline(tfull_bar(b), ph, abort_flag))) return false;
           tc_fence_after();
-          const uint32_t acc = tmem + lane_addr + b * (uint32_t)stride;
+          const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + b * (uint32_t)stride;
           // the accumulator is free once its scores are in registers: the MMA issuer does not wait for what follows
           const uint32_t free_bar = tempty_bar(b);
           next_acc();
@@ -628,46 +618,49 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
             mask = ~mask;
             const int left = qn - 32 * part;   // padding queries past qn are never admitted
             if (left < 32) mask &= (1u << left) - 1u;
-            const uint32_t j = entry(r);
+            const uint32_t j = entry(t0 + r);
             const uint32_t full = j < j_end ? push(mask, j) : 0u;
             if (full) {
-              over |= 1u << r;
+              rest[kRound] |= 1u << r;
               rest[r] = full;
             }
             __syncwarp();   // the next load is warp-collective
           }
         }
-        // close the queue while it is past kFlushAt or a pair found it full, then queue the pairs that did (every
-        // turn either queues all of them or fills the queue, so this ends). All mask warps leave together.
-        for (;;) {
-          __syncwarp();
-          if (!mask_any(!got || *abort_flag || over != 0 || top >= kFlushAt)) break;
-          if (mask_any(!got || *abort_flag)) {
-            if (!got) fail();
-            stop = true;
+        return true;
+      };
+      // Whether the queue has to be closed now, with *last set after a timeout. All mask warps get the same answer.
+      auto must_close = [&](bool got, bool* last) -> bool {
+        __syncwarp();
+        if (!mask_any(!got || *abort_flag || *reinterpret_cast<volatile int*>(&t.count) > kFlushAt)) return false;
+        *last = mask_any(!got || *abort_flag);
+        if (!got) fail();
+        return true;
+      };
+      // close the queue (every mask warp has queued its pairs); the pass's last close also after a timeout: the checkers
+      // leave only at a reopening
+      auto close = [&](bool last) {
+        if (threadIdx.x == 0) {
+          if (last) t.pass_end = 1;
+          st_volatile(&t.closed, 1u + (uint32_t)min(t.count, kCap));
+        }
+      };
+
+      if (warp < kMaskWarps) {
+        rest[kRound] = 0;
+        first_acc(it);
+        bool last = true;
+        for (uint32_t t0 = 0; t0 < nb; t0 += kRound)
+          if (must_close(scan_round(t0), &last)) {
+            rest[kRound + 1] = t0;
             break;
           }
-          close(false);
-          reopen(t, mw, lane);   // once the checkers are done with it
-          ++ep;
-          top = -1;
-          for (uint32_t o = over; o; o &= o - 1) {
-            const int i = __ffs(o) - 1;
-            rest[i] = push(rest[i], entry(i));
-            if (!rest[i]) over &= ~(1u << i);
-          }
-        }
+        close(last);
       }
-      // the pass's last close, also after a timeout: the checkers leave only at a reopening
-      close(true);
-    }
-
-    if (warp < kEpiWarps) {
-      // ---------------- checker warps, and the mask warps once the range is scanned ----------------
-      // claim a queue position (several for narrow rows), check and fold its pair while the scan goes on; at a close,
-      // finish what was queued below it, then take part in the reopening
-      const int claims = a.d <= 256 ? kNarrowItems : 1;
-      for (;;) {
+      for (;;) {   // an epoch of the queue
+        // claim a queue position (several for narrow rows), check and fold its pair while the scan goes on; at a close,
+        // finish what was queued below it, then take part in the reopening
+        const int claims = a.d <= 256 ? kNarrowItems : 1;
         for (;;) {
           int base = 0;
           if (lane == 0) base = atomicAdd(&t.claim, claims);
@@ -695,6 +688,30 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
         const bool end = reopen(t, warp, lane);
         ++ep;
         if (end) break;
+        if (warp < kMaskWarps) {
+          // The range's rest: first what found the queue full (every epoch either queues all of it or fills the queue, so this
+          // ends). A copy of the scan above and no way back to it, which would keep more in registers over the checks: the
+          // common pass, with one close, then spills (8 % of a lookup).
+          uint32_t t0 = rest[kRound + 1], left = 0;
+          for (uint32_t o = rest[kRound]; o; o &= o - 1) {
+            const int i = __ffs(o) - 1;
+            rest[i] = push(rest[i], entry(t0 + i));
+            if (rest[i]) left |= 1u << i;
+          }
+          rest[kRound] = left;
+          t0 += kRound;
+          first_acc(it + min(t0, nb));
+          bool last = true;
+          for (bool got = true; !must_close(got, &last); t0 += kRound) {
+            if (t0 >= nb) {
+              last = true;
+              break;
+            }
+            got = scan_round(t0);
+          }
+          rest[kRound + 1] = t0 - kRound;
+          close(last);
+        }
       }
     }
 

@@ -253,12 +253,29 @@ def test_large_stores_take_the_tensor_scan_earlier_and_equal_the_exact_scan(n, b
     assert np.array_equal(a["entry_id"][hit], b["entry_id"][hit])
 
 
+def test_tensor_scan_goes_on_after_the_queue_filled_up():
+    # 72 blocks per CTA in rounds of 32, a pass of 128 queries and one of 3, every pair admitted: each round fills the queue
+    # over and over, and the scan goes on after it, with whole and ragged rounds and an idle column chunk
+    w = wl.WORKLOADS["mid-1m"].scaled(n=1_400_001, d=64, batch=131, clusters=5_000)
+    with new_cache(w, L.LACACHE_STAGE1_TENSOR) as exact_cache, new_cache(w, L.LACACHE_STAGE1_LSH) as cache:
+        for c in (exact_cache, cache):
+            fill(c, w)
+        L.lacache_enable_lsh(cache.h, 128, 128, wl.hyperplanes(128, w.d, device="cuda"))
+        q = wl.batch(w, 0, device="cuda")
+        a, b = gpu_lookup(exact_cache, q), gpu_lookup(cache, q)
+        assert cache.last_launch()[1] == L.LACACHE_STAGE1_LSH_TENSOR
+    # fp32 sums of 64 products of bf16 unit rows in two orders: |difference| <= 64 * 2^-24 * sum |x y| < 4e-6
+    assert np.array_equal(a["n_cand"], b["n_cand"]) and np.array_equal(a["status"], b["status"])
+    assert np.allclose(a["key_score"], b["key_score"], rtol=0, atol=4e-6)
+    assert np.allclose(a["cand_score"], b["cand_score"], rtol=0, atol=4e-6, equal_nan=True)
+
+
 @pytest.mark.slow
 def test_a_long_drain_of_the_queue_is_not_a_timeout():
     # radius = bits on 48 blocks of 128 rows per CTA: a round of 32 blocks leaves 524,288 pairs to a queue of 4,096. Rows
     # of 8,192 elements whose scores rise along each CTA's range, so that every pair enters a list of 32, make their
-    # checks take 0.8 s, and for that long the loader, the expanders and the MMA issuer stand still: nearly the budget of
-    # one wait, which has to count the drain's progress
+    # checks take a quarter of a second (0.8 s when the checker warps did them alone), and for that long the loader, the
+    # expanders and the MMA issuer stand still. The budget of their waits, a second, has to count the drain's progress.
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     per, d, batch, bits, top_c, chunk = 48 * 128, 8192, 128, 256, 32, 1 << 15
     n = per * sms
