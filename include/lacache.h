@@ -198,7 +198,8 @@ lacache_status lacache_append_misses(lacache_t* h, int32_t B, const void* q_emb_
  * differs from the query's in at most `radius` bits; stage 2 is unchanged. Existing entries are signed now and
  * later inserts and appends are signed as they arrive. Batches of fewer than T queries compare the packed
  * signatures by population counts; larger ones run the Hamming test on the tensor cores. T = 48 at 256 bits and 40 at
- * 128 and 512; on stores of 131,072 entries and more 33; from 2,097,152 entries 32, 24 and 18 at 128, 256 and 512 bits.
+ * 128 and 512; on stores of 131,072 entries and more 33, and from 2,097,152 entries 32, 24 and 18 at 128, 256 and 512
+ * bits, unless the radius is so wide that at least a tenth of an unrelated pair per entry is expected within it.
  * Allocates (capacity + max_batch) * bits / 8 bytes for the signatures.
  * Asynchronous on cuda_stream; calling it again replaces the index. A lookup on a handle whose cfg->stage1 is
  * LACACHE_STAGE1_LSH returns LACACHE_ERR_INVALID_ARG, and runs nothing, until this call has been made. */

@@ -46,6 +46,7 @@ struct lacache {
   int64_t lookups, queries, inserted, appended;   // host-side counters
   int lsh_bits;              // SimHash index: signature bits (0 = no index)
   int lsh_radius;
+  double lsh_unrelated;      // the share of unrelated pairs within the radius (random_pair_within)
   uint32_t* sig;             // [capacity x lsh_bits/32] entry signatures (one allocation with qsig and hyper)
   uint32_t* qsig;            // [max_batch x lsh_bits/32] query signatures of the current lookup
   __nv_bfloat16* hyper;      // [lsh_bits x d] hyperplanes
@@ -452,7 +453,7 @@ lacache_status run_lookup(lacache* h, int32_t B, const void* q_emb, const void* 
               : lc::launch_sign_queries(a.q, B, c.d, h->hyper, h->lsh_bits, h->qsig, st, gathered);
       if (e == cudaSuccess) {
         lc::LshArgs l{h->sig, h->qsig, h->lsh_bits / 32, h->lsh_radius};
-        if (B >= lc::lsh_tensor_min_batch(h->lsh_bits, h->n)) {
+        if (lc::lsh_takes_tensor(h->lsh_bits, h->lsh_unrelated, h->n, B)) {
           e = lc::launch_stage1_lsh_tc(a, l, h->num_sms, h->max_splits, st, &splits);
           kernel = LACACHE_STAGE1_LSH_TENSOR;
           if (a.inject_stall) --h->inject_stall;
@@ -842,6 +843,7 @@ lacache_status lacache_enable_lsh(lacache_t* h, int32_t bits, int32_t radius, co
   h->hyper = reinterpret_cast<__nv_bfloat16*>(h->qsig + qsig_bytes / 4);
   h->lsh_bits = bits;
   h->lsh_radius = radius;
+  h->lsh_unrelated = lc::random_pair_within(bits, radius);
   if (cudaMemcpyAsync(h->hyper, hyperplanes_dev, (size_t)bits * c.d * 2, cudaMemcpyDeviceToDevice, st) !=
           cudaSuccess ||
       sign_rows(h, 0, h->n, st) != cudaSuccess)

@@ -516,14 +516,6 @@ bool bulk_ring(int words, int B, int64_t n, int splits) {
   return words == 16 || (B == 1 && n / splits >= 16 * (int64_t)kTile);
 }
 
-// Probability that two independent uniformly random n-bit strings differ in at most r positions.
-double random_pair_within(int n, int r) {
-  if (r >= n) return 1.0;
-  double p = 0.0;
-  for (int i = 0; i <= r; ++i) p += std::exp(std::lgamma(n + 1.0) - std::lgamma(i + 1.0) - std::lgamma(n - i + 1.0));
-  return p * std::exp(-n * std::log(2.0));
-}
-
 // The distance test's prefix: 3, 5 or 8 words at W = 4, 8 or 16 (96, 160 or 256 bits) when at most 2 % of
 // unrelated pairs (whose distance is about that of random strings) stay within the radius on it, else the whole
 // signature. At the radii the thresholds give (35, 60 and 106 bits at tau_c = 0.9) the prefix keeps 0.5 %, 0.1 %
@@ -548,6 +540,13 @@ cudaError_t launch_form(bool bulk, const Stage1Args& a, const LshArgs& l, int sp
 }
 
 }  // namespace
+
+double random_pair_within(int n, int r) {
+  if (r >= n) return 1.0;
+  double p = 0.0;
+  for (int i = 0; i <= r; ++i) p += std::exp(std::lgamma(n + 1.0) - std::lgamma(i + 1.0) - std::lgamma(n - i + 1.0));
+  return p * std::exp(-n * std::log(2.0));
+}
 
 cudaError_t launch_sign_queries(const __nv_bfloat16* q, int B, int d, const __nv_bfloat16* hyperplanes, int bits,
                                 uint32_t* qsig, cudaStream_t st, bool q_from_previous) {

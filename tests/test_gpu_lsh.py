@@ -301,3 +301,24 @@ def test_a_long_drain_of_the_queue_is_not_a_timeout():
     # an fp32 sum of 8,192 products of unit rows: within 8192 * 2^-24 * sum |x y| < 5e-4 of the exact one
     best = float(key[-1].double() @ u.bfloat16().double())
     assert np.allclose(got["key_score"], best, rtol=0, atol=5e-4)
+
+
+@pytest.mark.parametrize("bits,batch,radius,kernel", [(128, 33, 48, L.LACACHE_STAGE1_LSH_TENSOR), (128, 33, 49, L.LACACHE_STAGE1_LSH),
+                                                      (128, 39, 64, L.LACACHE_STAGE1_LSH), (128, 40, 64, L.LACACHE_STAGE1_LSH_TENSOR),
+                                                      (256, 47, 112, L.LACACHE_STAGE1_LSH), (512, 33, 512, L.LACACHE_STAGE1_LSH)])
+def test_wide_radii_keep_the_switch_of_small_stores(bits, batch, radius, kernel):
+    # both sides of the radius and of the batch at which lookups on 131,072 entries go to the tensor-core scan: 33 queries
+    # admit 0.098 unrelated pairs per entry at radius 48 of 128 bits and 0.17 at 49. Every radius here keeps all candidates
+    # (test_large_stores_take_the_tensor_scan_earlier_and_equal_the_exact_scan), so the lookup is the exact scan's
+    w = wl.WORKLOADS["mid-1m"].scaled(n=131_072, d=64, batch=batch)
+    with new_cache(w, L.LACACHE_STAGE1_TENSOR) as exact_cache, new_cache(w, L.LACACHE_STAGE1_LSH) as cache:
+        for c in (exact_cache, cache):
+            fill(c, w)
+        L.lacache_enable_lsh(cache.h, bits, radius, wl.hyperplanes(bits, w.d, device="cuda"))
+        q = wl.batch(w, 0, device="cuda")
+        a, b = gpu_lookup(exact_cache, q), gpu_lookup(cache, q)
+        assert cache.last_launch()[1] == kernel
+    hit = a["status"] == L.LACACHE_HIT
+    assert hit.any()
+    assert np.array_equal(a["status"], b["status"]) and np.array_equal(a["n_cand"], b["n_cand"])
+    assert np.array_equal(a["entry_id"][hit], b["entry_id"][hit])
