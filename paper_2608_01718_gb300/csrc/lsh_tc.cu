@@ -36,7 +36,7 @@
 // CTA records LACACHE_ERR_DEVICE_TIMEOUT in the status word, the roles stop at the next pass boundary, in-flight
 // copies and MMAs are drained, TMEM is freed and the CTA exits.
 //
-// What bounds it: instruction issue (0.67 a scheduler and cycle at 128 queries and 256 bits, ALU pipe half busy), at
+// What bounds it: instruction issue (0.62 a scheduler and cycle at 128 queries and 256 bits, ALU pipe half busy), at
 // some 1,500 cycles per block of 128 entries at 128 queries; the packed index takes 20 us of HBM time on 4M entries,
 // the MMAs 55 us. So the warps' loops are kept short, and in 64 registers a thread almost without spills (32-bit entry
 // numbers, no running counts: 8 % at 128 queries); two expander sets, since one took 1,000 cycles a block and the MMAs
