@@ -392,11 +392,18 @@ int stage1_of(const lacache* h, int32_t B) {
 
 // Whether the kernels of a host-buffer lookup read its inputs (device addresses of mapped host memory) where they are,
 // without the gather: for the streaming scan, each of whose CTAs reads the batch once, while that is at most
-// kDirectBytes over the link in all; the tensor scan reads the batch again for every key tile.
-constexpr size_t kDirectBytes = (size_t)1 << 20;
-bool reads_host_inputs(const lacache* h, int32_t B, const void* emb, const void* pre, const void* ids) {
+// kDirectBytes over the link on all SMs; the tensor scan reads the batch again for every key tile. A call that is waited for
+// (`alone`) also sees how long the link takes: there at most kDirectBytesAlone by the CTAs that the store can give work
+// (one per 32 keys, a key tile of two for each of a CTA's warps). Measured (us a call, gathered / in place), waited for: 10,000 x
+// 768, 1 query 35.5 / 33.9, 2 (456 KB) 36.9 / 36.2, 4 (912 KB) 39.3 / 41.5; 10,000 x 128, 12 queries (456 KB) 42.5 / 41.7,
+// 16 (608 KB) 43.9 / 44.5; 1,000 x 768, 4 queries 35.9 / 33.4. Several in flight: 10,000 x 768, 4 queries 16.6 / 14.8; 10,000
+// x 128, 16 queries 21.2 / 18.6.
+constexpr size_t kDirectBytes = (size_t)1 << 20, kDirectBytesAlone = (size_t)1 << 19;
+bool reads_host_inputs(const lacache* h, int32_t B, const void* emb, const void* pre, const void* ids, bool alone) {
+  const size_t batch = (size_t)B * h->cfg.d * 2;
+  const size_t ctas = (size_t)std::min<int64_t>(h->num_sms, (h->n + 31) / 32);
   return stage1_of(h, B) == LACACHE_STAGE1_STREAM && emb && pre && ids && aligned16(emb) && aligned16(pre) &&
-         (uintptr_t)ids % 4 == 0 && (size_t)h->num_sms * B * h->cfg.d * 2 <= kDirectBytes;
+         (uintptr_t)ids % 4 == 0 && h->num_sms * batch <= kDirectBytes && (!alone || ctas * batch <= kDirectBytesAlone);
 }
 
 // Where a lookup's inputs come from: the caller's device memory, the staging that gather_host_kernel just wrote (so the
@@ -681,7 +688,7 @@ lacache_status lacache_lookup_host(lacache_t* h, int32_t B, const void* q_emb_ho
   const void* src[3];
   for (int i = 0; i < 3; ++i) src[i] = mapped_device_pointer(in.src[i]);
   Inputs inputs = Inputs::kDevice;
-  if (reads_host_inputs(h, B, src[0], src[1], src[2])) {
+  if (reads_host_inputs(h, B, src[0], src[1], src[2], true)) {
     inputs = Inputs::kHost;
   } else {
     next_stage_slot(h);
@@ -763,7 +770,7 @@ lacache_status lacache_lookup_host_async(lacache_t* h, int32_t B, const void* q_
                       map_output(o.cand_prefix_scores, &dev.cand_prefix_scores);
   if (!mapped) return LACACHE_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  if (reads_host_inputs(h, B, src[0], src[1], src[2]))
+  if (reads_host_inputs(h, B, src[0], src[1], src[2], false))
     return run_lookup(h, B, src[0], src[1], static_cast<const int32_t*>(src[2]), dev, st, Inputs::kHost);
   next_stage_slot(h);
   if (launch_gather(h, g, gathered, st) != cudaSuccess) return LACACHE_ERR_CUDA;

@@ -624,7 +624,7 @@ def test_append_takes_the_non_hit_rows_in_query_order(B):
 @pytest.mark.parametrize("d,batch", [(768, 1), (768, 4), (768, 5), (1024, 3), (1280, 2), (392, 7)])
 def test_host_lookups_read_small_batches_in_place(d, batch):
     # streaming-scan lookups from mapped pinned memory: batches of at most 1 MiB over all SMs (4 queries at d = 768, 3 at
-    # 1024, 8 at 392) are read where they are, others gathered first. The same buffers are refilled between calls, so a
+    # 1024, 8 at 392), half of it in the synchronous form, are read where they are, others gathered first. The same buffers are refilled between calls, so a
     # stale cache line would show; three lookups are in flight in the asynchronous form.
     w = wl.WORKLOADS["mid-1m"].scaled(n=9_000, d=d, batch=batch, clusters=90)
     with new_cache(w, L.LACACHE_STAGE1_STREAM) as cache:
@@ -679,9 +679,9 @@ def test_host_lookups_right_after_an_fp32_insert_see_its_rows(stage1, batch):
                                               (16, True, 16), (32, False, 5), (32, True, 40)])
 def test_in_place_host_lookups_for_every_list_size_and_ensembles(top_c, ensemble, k):
     # the second stage that stages its query in shared memory, for every list size (4, 8, 16 and 32 slots), one check and
-    # an ensemble of three (prefix rows of 2,176 elements), token ids past one warp's first 32. A batch of 3 at d = 768 is
+    # an ensemble of three (prefix rows of 2,176 elements), token ids past one warp's first 32. A batch of 2 at d = 768 is
     # read in place on the streaming scan; the device lookup of the same queries is the reference, bit for bit.
-    w = wl.WORKLOADS["ensemble-1m" if ensemble else "mid-1m"].scaled(n=9_000, batch=3, clusters=30, top_c=top_c, k=k)
+    w = wl.WORKLOADS["ensemble-1m" if ensemble else "mid-1m"].scaled(n=9_000, batch=2, clusters=30, top_c=top_c, k=k)
     with new_cache(w, L.LACACHE_STAGE1_STREAM) as cache:
         fill(cache, w)
         for step in range(3):
