@@ -64,7 +64,10 @@ __device__ __forceinline__ void keep(uint64_t (&loc)[CPAD], uint64_t x) {
 // before the wait for the grids ahead, and past the caches: the host may have written them since an earlier grid read
 // them.
 template <int CPAD, int kWarps, bool kHost>
-__global__ void __launch_bounds__(kWarps * 32, (kWarps == 8 ? 1 : 2) * (CPAD <= 8 ? 4 : CPAD <= 16 ? 3 : 2))
+__global__ void __launch_bounds__(kWarps * 32, kWarps == 8 && CPAD <= 4 ? 5
+                                                                        : (kWarps == 8 ? 1 : 2) * (CPAD <= 8    ? 4
+                                                                                                   : CPAD <= 16 ? 3
+                                                                                                                : 2))
     stage2_kernel(Stage2Args a) {
   constexpr int kThreads = kWarps * 32;
   extern __shared__ uint4 smem_q[];             // kHost: the query's prefix row [pd bf16], then its token ids [k]
@@ -274,6 +277,8 @@ cudaError_t launch_cpad(const Stage2Args& a, cudaStream_t st) {
 // alone (us, eight / four warps): 262,144 entries, top_c = 8, 512 queries 13.8 / 15.8, 1,024 19.3 / 16.9, 8,192 90 / 66;
 // 1M entries, top_c = 16, 512 queries 22.9 / 26.5, 1,024 35.9 / 31.9, 8,192 230 / 195 (295 with 87 registers a thread).
 constexpr int kLargeBatch = 1024;
+// Eight warps with lists of up to 4 stay at 48 registers a thread, so that three of their CTAs fit beside the next lookup's
+// stage 1 on an SM (with 64, two; 16,483 x 64, a lookup of 384 queries 21.4 us / 19.7, of 512 22.6 / 21.4).
 
 template <int CPAD>
 cudaError_t launch_warps(const Stage2Args& a, cudaStream_t st) {
