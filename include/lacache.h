@@ -280,9 +280,10 @@ lacache_status lacache_stage_times(lacache_t* h, double* stage1_ms, double* stag
  * thread's bounded wait for that tile runs out, the CTA still ends its passes and waits (bounded) for its issued
  * copies. The timeout is recorded the same way.
  * On CTA pairs the first CTA is the leader of the first pair; its abort stops its peer too. A single query tile
- * (B <= 128) runs on a dynamic schedule whose first tile is the CTA's own. What is withheld is its second load, so the
- * stall is certain for rows of more than 64 elements (two loads a tile); for shorter rows the first CTA has to claim a
- * second tile, which is certain when the store holds many more key tiles than the GPU has SMs. 0 cancels. */
+ * (B <= 128) runs on a dynamic schedule whose first tile is the CTA's own with top_c <= 16. What is withheld is its
+ * second load, so the stall is then certain for rows of more than 64 elements (two loads a tile); otherwise the first
+ * CTA has to claim a tile, or a second one, which is certain when the store holds many more key tiles than the GPU has
+ * SMs. 0 cancels. */
 lacache_status lacache_inject_stall(lacache_t* h, int32_t lookups);
 
 /* Lookup that allocates nothing, for callers that cannot allocate device memory. Examples: a serving runtime or

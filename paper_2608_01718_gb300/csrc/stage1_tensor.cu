@@ -336,12 +336,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         return true;
       };
       if (dyn) {
-        // the first tile is the CTA's own: no round trip to the counter before the first load
-        int64_t next = blockIdx.x;
+        // The first tile is the CTA's own: no round trip to the counter before the first load. Not with lists of more than 16:
+        // this kernel's registers and those of the stage 2 of the lookup before then don't fit one SM, and a CTA that
+        // starts only when that stage 2 ends must find no tile waiting for it (257,793 x 192, 22 queries, lists of 32: 31.1
+        // us a lookup with a first tile of its own, 27.6 without; 100,000 x 64, 32 queries 43.4 / 34.9. Lists of 8, 60,000 x
+        // 768, 32 queries: 18.9 / 19.4).
+        constexpr bool kOwnFirst = CPAD <= 16;
+        const int64_t own = kOwnFirst ? gridDim.x : 0;
+        int64_t next = kOwnFirst ? (int64_t)blockIdx.x : (int64_t)atomicAdd(p.tile_ctr, 1);
         for (uint32_t r = 0; ok; ++r) {
           const int64_t t = next;
           const bool done = t >= p.n_tiles;
-          if (!done) next = (int64_t)gridDim.x + atomicAdd(p.tile_ctr, 1);   // one ahead: hides the atomic's latency
+          if (!done) next = own + atomicAdd(p.tile_ctr, 1);   // one ahead: hides the atomic's latency
           const int slot = r % RING;
           if (!mbar_wait(tid_empty_bar(slot), ((r / RING) & 1u) ^ 1u, abort_flag)) {
             fail();
