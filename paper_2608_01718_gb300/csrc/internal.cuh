@@ -177,13 +177,13 @@ cudaError_t launch_stage1_lsh_tc(const Stage1Args& a, const LshArgs& l, int num_
 // So the lines below kLshLargeStore are on the popcount scan's side of the crossing: at 32 queries on 1M entries it is
 // 7 us behind at 256 bits and 17 at 512, further just below 2M, where its time has doubled, and 5 us at 40 queries on
 // 100,000 entries at 256 bits. The GPU tests expect it there (32 queries on 1M entries are its full-size case).
-// All that holds for radii that admit few pairs beside the near ones. Where the radius also admits unrelated ones, at `unrelated`
-// of them (random_pair_within), both scans spend their time on the exact checks, and the popcount scan, with 32 warps an SM
-// for them, does more at a time. So from a tenth of a pair per entry of the store the lines of small stores hold.
-// Measured (popcount / tensor, us): 1M x 64, 128 bits, 33 queries at radius 45 (0.02 pairs per entry) 76 / 73, 56 (3.0) 678 / 919,
-// 59 (7.0) 1,107 / 1,567; 256 bits, 33 at 105 (0.08) 237 / 263, 47 at 112 (1.2) 727 / 952; 2.2M x 64, 512 bits, 24 at 224 (0.06)
-// 689 / 808; 2.2M x 768, 128 bits, 32 at 56 2,122 / 2,558. (Between 0.03 and 0.1 the tensor scan is up to 15 % behind: the GPU
-// tests expect it at 0.098.)
+// All that holds for radii that admit few pairs beside the near ones. Where the radius also admits unrelated ones, at
+// `unrelated` of them (random_pair_within), both scans spend their time on the exact checks, and the popcount scan, with
+// 32 warps an SM for them, does more at a time. So from a tenth of a pair per entry of the store the lines of small stores
+// hold. Measured (popcount / tensor, us): 1M x 64, 128 bits, 33 queries at radius 45 (0.02 pairs per entry) 76 / 73, 56
+// (3.0) 678 / 919, 59 (7.0) 1,107 / 1,567; 256 bits, 33 at 105 (0.08) 237 / 263, 47 at 112 (1.2) 727 / 952; 2.2M x 64, 512
+// bits, 24 at 224 (0.06) 689 / 808; 2.2M x 768, 128 bits, 32 at 56 2,122 / 2,558. (Between 0.03 and 0.1 the tensor scan is
+// up to 15 % behind: the GPU tests expect it at 0.098.)
 constexpr int64_t kLshLargeStore = 1 << 21, kLshSecondPassStore = 1 << 17;
 constexpr double kLshWidePairs = 0.1;
 inline bool lsh_takes_tensor(int bits, double unrelated, int64_t n, int B) {

@@ -585,10 +585,11 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
         }
         return full;
       };
-      const auto entry = [&](uint32_t block) { return j_begin + block * kBlockRows + quad * 32 + lane; };   // this thread's
-      // A round: the blocks from t0 on, at most kRound. False after a timeout. Admitted pairs are rare: a first look at a block
-      // takes only the maximum of the chunk's scores; the admitted queries are told apart, and queued for the checker
-      // warps, where some lane's maximum reaches the threshold.
+      // this thread's entry of a block
+      const auto entry = [&](uint32_t block) { return j_begin + block * kBlockRows + quad * 32 + lane; };
+      // A round: the blocks from t0 on, at most kRound. False after a timeout. Admitted pairs are rare: a first look at a
+      // block takes only the maximum of the chunk's scores; the admitted queries are told apart, and queued for the
+      // checker warps, where some lane's maximum reaches the threshold.
       auto scan_round = [&](uint32_t t0) -> bool {
 #pragma unroll 1
         for (int r = 0; part < first_chunks && r < kRound && t0 + r < nb; ++r) {
@@ -689,9 +690,9 @@ __global__ void __launch_bounds__(kThreads, 1) lsh_tc_kernel(Stage1Args a, LshAr
         ++ep;
         if (end) break;
         if (warp < kMaskWarps) {
-          // The range's rest: first what found the queue full (every epoch either queues all of it or fills the queue, so this
-          // ends). A copy of the scan above and no way back to it, which would keep more in registers over the checks: the
-          // common pass, with one close, then spills (8 % of a lookup).
+          // The range's rest: first what found the queue full (every epoch either queues all of it or fills the queue, so
+          // this ends). A copy of the scan above and no way back to it, which would keep more in registers over the
+          // checks: the common pass, with one close, then spills (8 % of a lookup).
           uint32_t t0 = rest[kRound + 1], left = 0;
           for (uint32_t o = rest[kRound]; o; o &= o - 1) {
             const int i = __ffs(o) - 1;

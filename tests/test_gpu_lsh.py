@@ -303,10 +303,9 @@ def test_a_long_drain_of_the_queue_is_not_a_timeout():
     assert np.allclose(got["key_score"], best, rtol=0, atol=5e-4)
 
 
-@pytest.mark.parametrize("bits,batch,radius,kernel", [(128, 33, 48, L.LACACHE_STAGE1_LSH_TENSOR), (128, 33, 49, L.LACACHE_STAGE1_LSH),
-                                                      (128, 39, 64, L.LACACHE_STAGE1_LSH), (128, 40, 64, L.LACACHE_STAGE1_LSH_TENSOR),
-                                                      (256, 47, 112, L.LACACHE_STAGE1_LSH), (512, 33, 512, L.LACACHE_STAGE1_LSH)])
-def test_wide_radii_keep_the_switch_of_small_stores(bits, batch, radius, kernel):
+@pytest.mark.parametrize("bits,batch,radius,tensor", [(128, 33, 48, True), (128, 33, 49, False), (128, 39, 64, False),
+                                                      (128, 40, 64, True), (256, 47, 112, False), (512, 33, 512, False)])
+def test_wide_radii_keep_the_switch_of_small_stores(bits, batch, radius, tensor):
     # both sides of the radius and of the batch at which lookups on 131,072 entries go to the tensor-core scan: 33 queries
     # admit 0.098 unrelated pairs per entry at radius 48 of 128 bits and 0.17 at 49. Every radius here keeps all candidates
     # (test_large_stores_take_the_tensor_scan_earlier_and_equal_the_exact_scan), so the lookup is the exact scan's
@@ -317,7 +316,7 @@ def test_wide_radii_keep_the_switch_of_small_stores(bits, batch, radius, kernel)
         L.lacache_enable_lsh(cache.h, bits, radius, wl.hyperplanes(bits, w.d, device="cuda"))
         q = wl.batch(w, 0, device="cuda")
         a, b = gpu_lookup(exact_cache, q), gpu_lookup(cache, q)
-        assert cache.last_launch()[1] == kernel
+        assert cache.last_launch()[1] == (L.LACACHE_STAGE1_LSH_TENSOR if tensor else L.LACACHE_STAGE1_LSH)
     hit = a["status"] == L.LACACHE_HIT
     assert hit.any()
     assert np.array_equal(a["status"], b["status"]) and np.array_equal(a["n_cand"], b["n_cand"])
